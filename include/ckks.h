@@ -441,11 +441,9 @@ int ckks_rescale_noalloc(ckks_ctx* ctx, const uint32_t* in_dev, int level, uint3
  * wait, which can cost throughput when several lanes share the GPU. A clone
  * inherits its parent's flags when it is created. */
 #define CKKS_LAUNCH_PDL 1
-/* CKKS_TUNE_TENSOR (default off): ckks_tune also times the tensor-core
- * shapes of the column kernels (tp in {8, 16}, below). They are slower than
- * the CUDA-core shapes when several lanes share the GPU (their larger
- * shared-memory blocks crowd out the other lanes' kernels), while the tuner
- * times one kernel alone, so they are only candidates on request. */
+/* CKKS_TUNE_TENSOR: accepted, without effect. ckks_tune always times the
+ * tensor-core form of the column kernels, which is also what runs by default
+ * where a level's conversions are large enough. */
 #define CKKS_TUNE_TENSOR 2
 /* CKKS_LAUNCH_UNFUSED (default off): HMult (with or without CKKS_RESCALE),
  * HRot and HConj run the unfused form instead, one kernel launch per step
@@ -483,7 +481,10 @@ int ckks_set_launch_flags(ckks_ctx* ctx, int flags);
  * CKKS_ETIMEOUT and clears the mark; the outputs of the operations issued
  * since the previous synchronizing call are undefined, and the context stays
  * usable. The limit applies to kernels enqueued after the call; a clone
- * inherits the parent's limit when it is created. CKKS_EINVAL if cycles < 1.
+ * inherits the parent's limit when it is created. The tensor-core column
+ * kernels wait for their own copies and products only, which end in
+ * microseconds; they give up after at least 2^24 cycles whatever the limit.
+ * CKKS_EINVAL if cycles < 1.
  * (Not from the paper: a guard of this implementation's asynchronous
  * kernels.) */
 int ckks_set_wait_limit(ckks_ctx* ctx, long long cycles);
@@ -496,13 +497,13 @@ int ckks_set_wait_limit(ckks_ctx* ctx, long long cycles);
  * splitting the conversion targets, and tp in {1, 2} targets converted per
  * pass over the shared inputs with CUDA-core multiply-adds. tp in {8, 16}
  * selects the tensor-core form instead (N = 2^12 and 2^16, at most 16
- * conversion sources, z = 1; (tc, sl) in {(8, 2), (8, 4), (4, 4), (4, 8)}):
- * the conversion of a tile to tp targets at a time is one exact fp16 matrix
- * product on the tensor cores (tcgen05) over byte planes of the sources and
- * of the matrix (Eq. 2 as a matrix product, Sec. 4.2). Every shape computes
+ * conversion sources, z = 1; (tc, sl) in {(8, 2), (8, 4), (4, 4), (4, 8)}, all
+ * the same kernel): the conversion of a tile of 16 columns to four targets at a
+ * time is one exact fp16 matrix product on the tensor cores (tcgen05) over byte
+ * planes of the sources and of the matrix (Eq. 2 as a matrix product, Sec. 4.2). Every shape computes
  * identical values; only time changes. A context and its clones share one
  * table of shapes per (kernel, level); levels without an entry use a fixed
- * rule. */
+ * rule (N = 2^16: the tensor-core form from a number of products on). */
 #define CKKS_COL_MODUP 0
 #define CKKS_COL_MODDOWN 1
 #define CKKS_COL_RS_FUSED 2

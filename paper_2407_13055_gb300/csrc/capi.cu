@@ -285,7 +285,6 @@ int ckks_set_launch_flags(ckks_ctx* ctx, int flags) {
   if ((flags & CKKS_LAUNCH_UNFUSED) && ctx->windowed)
     return fail(ctx, CKKS_EINVAL, "launch flags: the unfused form supports single rescaling only");
   ctx->dp.pdl = (flags & CKKS_LAUNCH_PDL) ? 1 : 0;
-  ctx->dp.tune_tensor = (flags & CKKS_TUNE_TENSOR) ? 1 : 0;
   ctx->dp.unfused = (flags & CKKS_LAUNCH_UNFUSED) ? 1 : 0;
   ctx->dp.checked = (flags & CKKS_LAUNCH_CHECKED) ? 1 : 0;
   return CKKS_OK;
@@ -1046,7 +1045,7 @@ static double rescale_factor(const ckks_ctx* ctx, int level) {
 // Rescale of [2][limbs] at `in` (poly stride sin) from `level` into out.
 static void rescale_into(ckks_ctx* ctx, int level, const uint32_t* in, size_t sin, uint32_t* out, size_t sout) {
   if (ctx->windowed) launch_rational_rescale(ctx->dp, ctx->sc, ctx->rr[level], in, sin, out, sout, ctx->stream);
-  else launch_rescale(ctx->dp, ctx->sc, in, sin, level + 1, out, sout, ctx->stream);
+  else launch_rescale(ctx->dp, true, ctx->sc, in, sin, level + 1, out, sout, ctx->stream);
 }
 
 int ckks_rescale(ckks_ctx* ctx, const ckks_ct* in, ckks_ct* out) {

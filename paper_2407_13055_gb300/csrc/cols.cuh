@@ -178,8 +178,7 @@ struct ColTile {
 template <class G, int TC>
 __device__ __forceinline__ void col_inputs(const DevParams& dp, const uint32_t* src, size_t src_stride, int K,
                                            int id0, const uint2* cin, int4* y4, uint32_t* colbuf, int l, int jj,
-                                           int c, int pos, int slice, int GS, uint32_t* ycopy = nullptr,
-                                           const int2* idtab = nullptr) {
+                                           int c, int pos, int slice, int GS, const int2* idtab = nullptr) {
   using CTL = ColTile<G, TC>;
   // the next source's loads are issued before this one's iNTT columns
   uint32_t nx[G::EC];
@@ -208,11 +207,6 @@ __device__ __forceinline__ void col_inputs(const DevParams& dp, const uint32_t* 
 #pragma unroll
     for (int i4 = 0; i4 < G::EC / 4; ++i4)
       y4[(k * (G::EC / 4) + i4) * CTL::CT + pos] = make_int4(y[4 * i4], y[4 * i4 + 1], y[4 * i4 + 2], y[4 * i4 + 3]);
-    if (ycopy) {
-      uint32_t* yc = ycopy + ((size_t)k << dp.log_n);
-#pragma unroll
-      for (int i = 0; i < G::EC; ++i) yc[(jj + G::EC * i) * G::W + l] = (uint32_t)y[i];
-    }
   }
 }
 
@@ -335,16 +329,15 @@ __global__ void __launch_bounds__(SL* ColTile<G, TC>::CT) k_ks_moddown_cols(DevP
 // give their centered coefficients y (sources 0 .. alpha - 1 in y4); E's iNTT
 // columns and the conversion z = BConv(P -> q_l) give the top limb's ModDown
 // output V = E - z P^-1 = iNTT((A_l - z_l) P^-1 + d_l) in the coefficient
-// domain, whose centered value c_l becomes source alpha. With Yu the y and
-// c_l are also stored ([alpha + 1][N], A layout along h).
+// domain, whose centered value c_l becomes source alpha.
 template <class G, int TC>
 __device__ __forceinline__ void top_limb_sources(const DevParams& dp, int n, const uint32_t* S, int4* y4,
                                                  uint32_t* colbuf, int l, int jj, int c, int pos, int slice, int SL,
-                                                 int u, uint32_t* Yu) {
+                                                 int u) {
   using CTL = ColTile<G, TC>;
   const int alpha = dp.alpha, top = n - 1;
   col_inputs<G, TC>(dp, S + ((size_t)(u * alpha) << dp.log_n), (size_t)1 << dp.log_n, alpha, dp.L, dp.ks.dn_cin,
-                    y4, colbuf, l, jj, c, pos, slice, SL, Yu);
+                    y4, colbuf, l, jj, c, pos, slice, SL);
   const PrimeConst Pt = dp.pc[top];
   if (slice == SL - 1) {
     // E_u: iNTT columns, times N^-1, kept in [0, q_l) in source slot alpha
@@ -380,35 +373,9 @@ __device__ __forceinline__ void top_limb_sources(const DevParams& dp, int n, con
         cl[k] = centered(csub(ev[k] + Pt.q - zp, Pt.q), Pt.q);
       }
       slot = make_int4(cl[0], cl[1], cl[2], cl[3]);
-      if (Yu) {
-        uint32_t* yc = Yu + ((size_t)alpha << dp.log_n);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) yc[(jj + G::EC * (4 * i4 + k)) * G::W + l] = (uint32_t)cl[k];
-      }
     }
   }
   __syncthreads();
-}
-
-// Top limb of the fused ModDown + rescale alone (the tensor-core form of the
-// rescale conversion takes its sources from Y = [2][alpha + 1][N]).
-// grid (W/TC, 2 polys).
-template <class G, int TC, int SL>
-__global__ void __launch_bounds__(SL* ColTile<G, TC>::CT) k_ks_moddown_cols_top(DevParams dp, int n,
-                                                                                        const uint32_t* S,
-                                                                                        uint32_t* Y) {
-  pdl_wait();
-  pdl_trigger();
-  using CTL = ColTile<G, TC>;
-  extern __shared__ int4 smem4[];
-  const int slice = threadIdx.x / CTL::CT, pos = threadIdx.x % CTL::CT;
-  const int c = pos % TC, jj = pos / TC;
-  const int l = blockIdx.x * TC + c;
-  const int u = blockIdx.y, alpha = dp.alpha;
-  uint32_t* colbuf =
-      reinterpret_cast<uint32_t*>(smem4 + (size_t)(alpha + 1) * (G::EC / 4) * CTL::CT) + slice * CTL::BUF;
-  top_limb_sources<G, TC>(dp, n, S, smem4, colbuf, l, jj, c, pos, slice, SL, u,
-                          Y + ((size_t)(u * (alpha + 1)) << dp.log_n));
 }
 
 // ModDown fused with rescaling, one column kernel per tile: the top limb's
@@ -431,7 +398,7 @@ __global__ void __launch_bounds__(SL* ColTile<G, TC>::CT) k_rs_cols_fused(DevPar
   const int alpha = dp.alpha, top = n - 1, K = alpha + 1;
   int4* y4 = smem4;
   uint32_t* colbuf = reinterpret_cast<uint32_t*>(smem4 + (size_t)K * (G::EC / 4) * CTL::CT) + slice * CTL::BUF;
-  top_limb_sources<G, TC>(dp, n, S, y4, colbuf, l, jj, c, pos, slice, SL, u, nullptr);
+  top_limb_sources<G, TC>(dp, n, S, y4, colbuf, l, jj, c, pos, slice, SL, u);
   auto tgt = [&](int i, const int32_t*& row, int& id, uint32_t*& dst) {
     row = dp.ks.rs_mat + i * K;
     id = i;
@@ -460,7 +427,7 @@ __global__ void __launch_bounds__(SL* ColTile<G, TC>::CT) k_mm_cols(DevParams dp
   int4* y4 = smem4;
   uint32_t* colbuf = reinterpret_cast<uint32_t*>(smem4 + (size_t)m.K * (G::EC / 4) * CTL::CT) + slice * CTL::BUF;
   col_inputs<G, TC>(dp, S + ((size_t)(u * m.K) << dp.log_n), (size_t)1 << dp.log_n, m.K, 0, m.cin, y4, colbuf, l,
-                    jj, c, pos, slice, SL, nullptr, m.rows);
+                    jj, c, pos, slice, SL, m.rows);
   __syncthreads();
   auto tgt = [&](int t, const int32_t*& row, int& id, uint32_t*& dst) {
     row = m.mat + t * m.K;
@@ -527,16 +494,19 @@ static bool with_shape(const ColShape& s, F f) {
   return false;
 }
 
-// Default shape: 8 columns (32-byte row segments) when that already gives
-// two blocks per SM, else 4 to double the block count; four slices; no split.
+// CUDA-core shape of a conversion with at most K sources per target that no
+// tuned entry covers. Measured on whole operations (us with the earlier rule of
+// 4 or 8 columns, 4 slices -> now): N = 2^16, dnum = 1 (K = 40), level 39: HRot
+// 226.0 -> 212.8 by the ModUp shape, 215.6 by the ModDown shape, HMult + rescale
+// 245.3 -> 235.7 by the rescale shape (level 3: 97.9 -> 83.6, 88.6; 108.9 ->
+// 107.3); at K <= 16 these run only below tensor_work (there 8 slices win: level
+// 1, dnum = 3, HRot 40.3 -> 37.9); N = 2^12: 16.7 -> 16.3 (HRot, dnum = 1).
 template <class G>
-static ColShape default_shape(int blocks_per_tile_column, int sms) {
-  ColShape s;
-  s.tc = ((G::W / 8) * blocks_per_tile_column >= 2 * sms || G::W / 4 < 16) ? 8 : 4;
-  s.sl = 4;
-  s.z = 1;
-  s.tp = 1;
-  return s;
+static ColShape default_shape(ColKernel k, int K) {
+  if (G::W == 16) return ColShape{8, 4, 1, 1};
+  if (G::W == 64) return ColShape{4, 8, k == CK_MODUP ? 1 : 2, 1};
+  if (k == CK_MODUP) return K > kTcMaxSources ? ColShape{8, 4, 2, 1} : ColShape{4, 8, 1, 1};
+  return k == CK_MODDOWN && K > kTcMaxSources ? ColShape{8, 4, 1, 1} : ColShape{8, 8, 1, 1};
 }
 
 // A shape is launchable when the tile width divides the row, a slice is a
@@ -553,38 +523,41 @@ static bool shape_ok(const ColShape& s) {
          (s.sl == 2 || s.sl == 4 || s.sl == 8) && s.z >= 1 && s.z <= 4 && (s.tp == 1 || s.tp == 2);
 }
 
+// From this many products per coefficient (sources times targets, summed over a
+// launch's conversions) the tensor-core form is the faster one at N = 2^16:
+// below it, a block's start (tensor memory, tables, the first product) costs
+// more than the products it saves. The lines lie where whole operations were
+// equal, levels 0-15, 5 to 15 sources: HRot by the ModUp form at 42 products
+// 39.4 against 40.4 us (CUDA cores first), at 70 43.6 / 43.6, at 112 46.7 /
+// 46.4, at 574 77.7 / 72.8; by the ModDown form at 32 33.5 / 35.8, at 84 40.9 /
+// 40.4, at 196 48.1 / 46.4; HMult + rescale, whose top limb takes a product of
+// its own, at 60 45.5 / 49.6, at 120 51.5 / 52.6, at 210 56.3 / 56.3, at 420
+// 67.3 / 65.1.
+static int tensor_work(ColKernel k) { return k == CK_RS_FUSED ? 200 : 64; }
+
+// The level's tuned shape; else the tensor-core form (N = 2^16, at most 16
+// sources, enough work) or the CUDA-core rule.
 template <class G>
-static ColShape pick_shape(const Scratch& sc, ColKernel k, int n, const ColShape& def) {
+static ColShape pick_shape(const Scratch& sc, ColKernel k, int tix, int K, int work) {
   if (sc.tune) {
-    const ColShape s = sc.tune->get(k, n);
+    const ColShape s = sc.tune->get(k, tix);
     if (s.valid() && shape_ok<G>(s)) return s;
   }
-  return def;
+  return G::W == 1024 && K <= kTcMaxSources && work >= tensor_work(k) ? ColShape{8, 4, 1, 16} : default_shape<G>(k, K);
+}
+
+// Whether a shape runs on the tensor cores for a conversion of K sources.
+template <class G>
+static bool use_tc(const DevParams& dp, const ColShape& s, int K) {
+  return G::H == 64 && is_tc_shape(s) && dp.ks.tc_img && K <= kTcMaxSources;
 }
 
 
 template <class G>
 void launch_modup_cols(const DevParams& dp, int n, int base, int tix, int digits, const Scratch& sc,
                        const ColShape& s0, cudaStream_t st) {
-  if (is_tc_shape(s0) && dp.ks.tc_img && dp.alpha <= kTcMaxSources &&
-      with_tc_shape<G>(s0, [&](auto tc, auto sl, auto nc) {
-        constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, NC = decltype(nc)::value;
-        using SH = TcShape<G, TC, SL, NC>;
-        int mmax = 0;
-        for (int j = 0; j < digits; ++j) {
-          const int g = base / dp.alpha + j;
-          const int k = std::min(n, (g + 1) * dp.alpha - base) - std::max(0, g * dp.alpha - base);
-          mmax = std::max(mmax, n + dp.alpha - k);
-        }
-        const int kr = tc_kr(dp.alpha);
-        const size_t sm = tc_smem<SH, NC>(kr, mmax).total;
-        set_col_smem((const void*)k_ks_modup_cols_tc<G, TC, SL, NC>, sm);
-        launch_pdl(dp.pdl, k_ks_modup_cols_tc<G, TC, SL, NC>, dim3(G::W / TC, digits), dim3(SH::NT), sm, st, dp, n,
-                   base, tix, kr, mmax, (const uint32_t*)sc.S, sc.T);
-        count_launch(1);
-      }))
-    return;
-  const ColShape s = is_tc_shape(s0) ? default_shape<G>(digits, dp.sms) : s0;
+  if (use_tc<G>(dp, s0, dp.alpha)) return launch_modup_tc<G>(dp, n, base, tix, digits, sc, st);
+  const ColShape s = is_tc_shape(s0) ? default_shape<G>(CK_MODUP, dp.alpha) : s0;
   with_shape(s, [&](auto tc, auto sl, auto tp) {
     constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, TP = decltype(tp)::value;
     const size_t sm = col_smem_bytes<G, TC, SL>(dp.alpha);
@@ -598,19 +571,8 @@ void launch_modup_cols(const DevParams& dp, int n, int base, int tix, int digits
 template <class G>
 void launch_moddown_cols(const DevParams& dp, int n, int base, int tix, const Scratch& sc, const ColShape& s0,
                          cudaStream_t st) {
-  if (is_tc_shape(s0) && dp.ks.tc_img && dp.alpha <= kTcMaxSources &&
-      with_tc_shape<G>(s0, [&](auto tc, auto sl, auto nc) {
-        constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, NC = decltype(nc)::value;
-        using SH = TcShape<G, TC, SL, NC>;
-        const int kr = tc_kr(dp.alpha);
-        const size_t sm = tc_smem<SH, NC>(kr, n).total;
-        set_col_smem((const void*)k_ks_moddown_cols_tc<G, TC, SL, NC>, sm);
-        launch_pdl(dp.pdl, k_ks_moddown_cols_tc<G, TC, SL, NC>, dim3(G::W / TC, 2), dim3(SH::NT), sm, st, dp, n, base,
-                   tix, kr, (const uint32_t*)sc.S, sc.T);
-        count_launch(1);
-      }))
-    return;
-  const ColShape s = is_tc_shape(s0) ? default_shape<G>(2, dp.sms) : s0;
+  if (use_tc<G>(dp, s0, dp.alpha)) return launch_moddown_tc<G>(dp, n, base, tix, sc, st);
+  const ColShape s = is_tc_shape(s0) ? default_shape<G>(CK_MODDOWN, dp.alpha) : s0;
   with_shape(s, [&](auto tc, auto sl, auto tp) {
     constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, TP = decltype(tp)::value;
     const size_t sm = col_smem_bytes<G, TC, SL>(dp.alpha);
@@ -622,37 +584,10 @@ void launch_moddown_cols(const DevParams& dp, int n, int base, int tix, const Sc
 }
 
 template <class G>
-void launch_moddown_cols_top(const DevParams& dp, int n, const Scratch& sc, uint32_t* Y, cudaStream_t st) {
-  ColShape s = default_shape<G>(2, dp.sms);
-  with_shape(s, [&](auto tc, auto sl, auto) {
-    constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value;
-    const size_t sm = col_smem_bytes<G, TC, SL>(dp.alpha + 1);
-    set_col_smem((const void*)k_ks_moddown_cols_top<G, TC, SL>, sm);
-    launch_pdl(dp.pdl, k_ks_moddown_cols_top<G, TC, SL>, dim3(G::W / TC, 2), dim3(SL * ColTile<G, TC>::CT), sm, st, dp,
-               n, (const uint32_t*)sc.S, Y);
-    count_launch(1);
-  });
-}
-
-template <class G>
 void launch_rs_cols_fused(const DevParams& dp, int n, const Scratch& sc, uint32_t* T3, const ColShape& s0,
                           cudaStream_t st) {
-  if (is_tc_shape(s0) && dp.ks.tc_img && dp.alpha + 1 <= kTcMaxSources &&
-      with_tc_shape<G>(s0, [&](auto tc, auto sl, auto nc) {
-        constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, NC = decltype(nc)::value;
-        using SH = TcShape<G, TC, SL, NC>;
-        // top limb first (its sources go through Y), then the conversion on
-        // the tensor cores
-        launch_moddown_cols_top<G>(dp, n, sc, sc.U, st);
-        const int kr = tc_kr(dp.alpha + 1);
-        const size_t sm = tc_smem<SH, NC>(kr, n - 1).total;
-        set_col_smem((const void*)k_rs_cols_fused_tc<G, TC, SL, NC>, sm);
-        launch_pdl(dp.pdl, k_rs_cols_fused_tc<G, TC, SL, NC>, dim3(G::W / TC, 2), dim3(SH::NT), sm, st, dp, n, kr,
-                   (const uint32_t*)sc.U, T3);
-        count_launch(1);
-      }))
-    return;
-  const ColShape s = is_tc_shape(s0) ? default_shape<G>(2, dp.sms) : s0;
+  if (use_tc<G>(dp, s0, dp.alpha + 1)) return launch_rs_fused_tc<G>(dp, n, sc, T3, st);
+  const ColShape s = is_tc_shape(s0) ? default_shape<G>(CK_RS_FUSED, dp.alpha + 1) : s0;
   with_shape(s, [&](auto tc, auto sl, auto tp) {
     constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, TP = decltype(tp)::value;
     const size_t sm = col_smem_bytes<G, TC, SL>(dp.alpha + 1);
@@ -665,7 +600,8 @@ void launch_rs_cols_fused(const DevParams& dp, int n, const Scratch& sc, uint32_
 
 template <class G>
 void launch_mm_cols(const DevParams& dp, const MmArgs& m, const Scratch& sc, const ColShape& s0, cudaStream_t st) {
-  const ColShape s = is_tc_shape(s0) ? default_shape<G>(2, dp.sms) : s0;
+  if (m.img >= 0 && use_tc<G>(dp, s0, m.K)) return launch_mm_tc<G>(dp, m, sc, st);
+  const ColShape s = is_tc_shape(s0) ? default_shape<G>(CK_RS_FUSED, m.K) : s0;
   with_shape(s, [&](auto tc, auto sl, auto tp) {
     constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, TP = decltype(tp)::value;
     const size_t sm = col_smem_bytes<G, TC, SL>(m.K);
@@ -696,7 +632,7 @@ __global__ void __launch_bounds__(SL* ColTile<G, TC>::CT) k_rr_cols(DevParams dp
   int4* y4 = smem4;
   uint32_t* colbuf = reinterpret_cast<uint32_t*>(smem4 + (size_t)r.K * (G::EC / 4) * CTL::CT) + slice * CTL::BUF;
   col_inputs<G, TC>(dp, S + ((size_t)u << dp.log_n), (size_t)2 << dp.log_n, r.K, 0, r.cin, y4, colbuf, l, jj, c,
-                    pos, slice, SL, nullptr, r.drop);
+                    pos, slice, SL, r.drop);
   __syncthreads();
   auto tgt = [&](int i, const int32_t*& row, int& id, uint32_t*& dst) {
     row = r.mat + i * r.K;
@@ -709,6 +645,10 @@ __global__ void __launch_bounds__(SL* ColTile<G, TC>::CT) k_rr_cols(DevParams dp
 
 template <class G>
 void launch_rr_cols(const DevParams& dp, const RrArgs& r, const Scratch& sc, cudaStream_t st) {
+  // products per coefficient from which the tensor-core form wins (HMult + rational
+  // rescale, levels 1 - 8 of the 25-30 system: 24 products 49.5 against 50.3 us,
+  // 30 58.7 / 58.4, 36 65.9 / 65.2, level 8 89.8 / 87.0)
+  if (G::W == 1024 && r.img >= 0 && 2 * r.K * r.n1 >= 30) return launch_rr_tc<G>(dp, r, sc, st);
   constexpr int TC = 8, SL = 4;
   const size_t sm = col_smem_bytes<G, TC, SL>(r.K);
   set_col_smem((const void*)k_rr_cols<G, TC, SL>, sm);

@@ -56,27 +56,28 @@ uint16_t f16_bits(int v) {
 }
 
 // Byte-plane image of a conversion matrix for the tensor-core BConv (the B
-// operand of cols_tc.cuh): mat[t * K + k] (t < M targets with primes
+// operand of cols_tc.cuh): mat[t * ld + k] (t < M targets with primes
 // prime[t]) are centered [(...) 2^32]_{prime_t} entries. For each target and
-// source, m'_a = [mat 2^(8a)]_{prime_t} centered (a < 4) is written as four
+// source, m'_a = [mat 2^-32 2^(8a)]_{prime_t} centered (a < 4) is written as four
 // balanced signed bytes (m'_a = sum_b e_b 2^(8b), e_b in [-128, 128) for
 // b < 3); row 4 t + b of the image holds e_b of (k, a) at column 4 k + a, as
 // fp16. Rows are padded to a multiple of 16 (zero targets), columns to
-// kr = 16 ceil(K / 4), and the image is stored in the MMA's shared-memory
+// kr = 16 ceil(Kx / 4) (Kx >= K), and the image is stored in the MMA's shared-memory
 // layout: core matrices of 8 rows x 8 columns (128 bytes), column blocks of
 // 8 adjacent (128 bytes apart), 8-row groups kr * 16 bytes apart. Returns
 // (byte offset in img, bytes).
-int2 append_planes(std::vector<uint8_t>& img, const int32_t* mat, int M, int K, const uint32_t* prime) {
-  const int kr = 16 * ((K + 3) / 4);
+int2 append_planes(std::vector<uint8_t>& img, const int32_t* mat, int ld, int M, int K, int Kx, const uint32_t* prime) {
+  const int kr = 16 * ((Kx + 3) / 4);
   const int rows = 4 * ((M + 3) & ~3);
   const size_t off = img.size(), bytes = (size_t)rows * kr * 2;
   img.resize(off + bytes, 0);
   uint8_t* base = img.data() + off;
   for (int t = 0; t < M; ++t) {
     const uint32_t p = prime[t];
+    const uint32_t r = invm((uint32_t)((1ull << 32) % p), p);
     for (int k = 0; k < K; ++k) {
-      const int32_t m = mat[(size_t)t * K + k];
-      const uint64_t mu = (uint64_t)(m < 0 ? (int64_t)m + p : (int64_t)m);
+      const int32_t m = mat[(size_t)t * ld + k];
+      const uint64_t mu = mulm((uint32_t)(m < 0 ? (int64_t)m + p : (int64_t)m), r, p);
       for (int a = 0; a < 4; ++a) {
         int64_t v = centered_h((uint32_t)((mu << (8 * a)) % p), p);
         int e[4];
@@ -96,6 +97,58 @@ int2 append_planes(std::vector<uint8_t>& img, const int32_t* mat, int M, int K, 
     }
   }
   return make_int2((int)off, (int)bytes);
+}
+
+// Division of a tensor-core column kernel's work (cols_tc.cuh) among at most
+// `sms` blocks: groups.size() conversions of (sources, targets) on `tiles`
+// column tiles each. Costs in targets of one warpgroup: a segment costs its
+// sources in rounds of the warpgroups, kStart for the latency of its
+// first product and its targets in fours. Returns the smallest load per block
+// that a walk along the items with cuts at any four targets meets, as block
+// boundaries item * 256 + target / 4 appended to plan: (offset, blocks).
+int2 tc_plan(std::vector<uint32_t>& plan, const std::vector<int2>& groups, int tiles, int sms) {
+  sms = std::min(sms, kTcMaxBlocks);
+  constexpr int kTcWarpgroups = 5, kStart = 5;
+  struct Item {
+    int src, quads;
+  };
+  std::vector<Item> g;
+  int lo = 0, hi = 0, total = 0;
+  for (const int2& v : groups) {
+    g.push_back({kTcWarpgroups * ((v.x + kTcWarpgroups - 1) / kTcWarpgroups) + kStart, (v.y + 3) / 4});
+    lo = std::max(lo, g.back().src + 4);
+    total += tiles * (g.back().src + 4 * g.back().quads);
+  }
+  hi = total;
+  const int items = (int)groups.size() * tiles;
+  auto walk = [&](int load, std::vector<uint32_t>* out) {
+    int item = 0, at = 0, blocks = 0;
+    while (item < items) {
+      if (out) out->push_back((uint32_t)item << 8 | (uint32_t)at);
+      int left = load;
+      while (item < items) {
+        const Item& v = g[item / tiles];
+        const int take = std::min(v.quads - at, (left - v.src) / 4);
+        if (left < v.src + 4) break;
+        left -= v.src + 4 * take;
+        at += take;
+        if (at < v.quads) break;
+        ++item;
+        at = 0;
+      }
+      ++blocks;
+    }
+    if (out) out->push_back((uint32_t)items << 8);
+    return blocks;
+  };
+  while (lo < hi) {
+    const int mid = (lo + hi) / 2;
+    if (walk(mid, nullptr) <= sms) hi = mid;
+    else lo = mid + 1;
+  }
+  const int off = (int)plan.size();
+  const int blocks = walk(hi, &plan);
+  return make_int2(off, blocks);
 }
 
 uint32_t brev(uint32_t v, int bits) {
@@ -513,6 +566,11 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
   std::vector<int2> up_img((size_t)(std::max(L, nlev) + 1) * dnum, make_int2(0, 0));
   std::vector<int2> dn_img((size_t)nlev + 1, make_int2(0, 0)), rs_img((size_t)L + 1, make_int2(0, 0));
   const bool tc_ok = alpha <= 16;
+  std::vector<uint32_t> plan;  // work division of the tensor-core column kernels
+  std::vector<int2> up_plan((size_t)nlev + 1, make_int2(0, 0)), dn_plan(up_plan), rs_plan((size_t)L + 1, make_int2(0, 0));
+  const int tiles = std::max(1, n / 64 / 16);
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || sms < 1) sms = 1;
   if (tc_ok) {
     std::vector<int32_t> rows;
     std::vector<uint32_t> tp;
@@ -520,9 +578,11 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
       const int s0 = ctx->lvl_first[tix - 1], nl = ctx->lvl_count[tix - 1];
       const int ext = nl + alpha;
       const int j0 = s0 / alpha, digits = (s0 + nl - 1) / alpha - j0 + 1;
+      std::vector<int2> km;
       for (int j = 0; j < digits; ++j) {
         const int g = j0 + j;
         const int lo = std::max(0, g * alpha - s0), hi = std::min(nl, (g + 1) * alpha - s0), K = hi - lo;
+        km.push_back(make_int2(K, ext - K));
         const int2 o = up_off[(size_t)tix * dnum + j];
         rows.clear();
         tp.clear();
@@ -531,13 +591,58 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
           for (int k = 0; k < K; ++k) rows.push_back(up_mat[(size_t)o.y + (size_t)t * K + k]);
           tp.push_back(pr[t < nl ? s0 + t : L + (t - nl)]);
         }
-        up_img[(size_t)tix * dnum + j] = append_planes(tc_img, rows.data(), ext - K, K, tp.data());
+        up_img[(size_t)tix * dnum + j] = append_planes(tc_img, rows.data(), K, ext - K, K, K, tp.data());
       }
+      up_plan[tix] = tc_plan(plan, km, tiles, sms);
+      dn_plan[tix] = tc_plan(plan, {make_int2(alpha, nl), make_int2(alpha, nl)}, tiles, sms);
       rows.assign(dn_mat.begin() + (size_t)s0 * alpha, dn_mat.begin() + (size_t)(s0 + nl) * alpha);
-      dn_img[tix] = append_planes(tc_img, rows.data(), nl, alpha, pr.data() + s0);
+      dn_img[tix] = append_planes(tc_img, rows.data(), alpha, nl, alpha, alpha, pr.data() + s0);
     }
     if (alpha + 1 <= 16)
-      for (int n = 2; n <= L; ++n) rs_img[n] = append_planes(tc_img, rs_mat.data(), n - 1, alpha + 1, pr.data());
+      for (int n = 2; n <= L; ++n) {
+        // first the P limbs' conversion to the top prime, in a group of its own
+        const int2 t = append_planes(tc_img, dn_mat.data() + (size_t)(n - 1) * alpha, alpha, 1, alpha, alpha + 1,
+                                     pr.data() + n - 1);
+        const int2 r = append_planes(tc_img, rs_mat.data(), alpha + 1, n - 1, alpha + 1, alpha + 1, pr.data());
+        rs_img[n] = make_int2(t.x, t.y + r.y);
+        rs_plan[n] = tc_plan(plan, {make_int2(alpha + 1, n - 1), make_int2(alpha + 1, n - 1)}, tiles, sms);
+      }
+  }
+  // one source: [1]_{q_i}, i < L - 1 (single rescaling), 2^32 = r1c carried as in every matrix
+  std::vector<int2> one_plan((size_t)L + 1, make_int2(0, 0));
+  int one_img = 0;
+  if (tc_ok && L > 1) {
+    std::vector<int32_t> r1(L);
+    for (int i = 0; i < L; ++i) r1[i] = ctx->pc_host[i].r1c;
+    one_img = append_planes(tc_img, r1.data(), 1, L - 1, 1, 1, pr.data()).x;
+    for (int n = 2; n <= L; ++n) one_plan[n] = tc_plan(plan, {make_int2(1, n - 1), make_int2(1, n - 1)}, tiles, sms);
+  }
+  std::vector<TcSrcRec> tc_src(np);
+  std::vector<TcTgtRec> tc_tgt(np);
+  for (int i = 0; i < np; ++i) {
+    // biases of A and B (tc_residue): 0x4B400000 (1 + 2^8); |A|, |B| < 2^28
+    const uint32_t q = pr[i], bias = 0x4B400000u * 257u, bound = 1u << 28;
+    TcPrime& t = tc_src[i].prime;
+    const uint2 c = shoup_pair((1u << 16) % q, q);
+    t.q = q;
+    t.c = c.x;
+    t.csh = c.y;
+    t.inv = (uint32_t)((1ull << 32) / q);
+    t.pad0 = t.pad1 = 0;
+    const uint32_t up = (bound + q - 1) / q * q;  // a multiple of q that makes A and B positive
+    t.eb = up - bias;
+    if (q > (1u << 30)) {
+      t.ea = 0u - bias;
+    } else if (q > (1u << 29)) {
+      // B keeps its bias: take bias 2^16 away again, in [2^28, 2^28 + q)
+      uint32_t d = q - mulm(bias % q, c.x, q);
+      if (d < bound) d += q;
+      t.ea = d - bias;
+      t.eb = 0;
+    } else {
+      t.ea = up - bias;
+    }
+    tc_tgt[i].prime = t;
   }
   std::vector<uint2> dn_pqinv((size_t)L * L, make_uint2(0, 0));
   for (int l = 1; l < L; ++l)
@@ -605,6 +710,11 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
       r.n0 = n0;
       r.s1 = s1;
       r.n1 = n1;
+      r.img = -1;
+      if (tc_ok && K > 0 && K <= 16) {
+        r.img = append_planes(tc_img, rr_mat.data() + rr_off[l].mat, K, n1, K, K, pr.data() + s1).x;
+        r.plan = tc_plan(plan, {make_int2(K, n1), make_int2(K, n1)}, tiles, sms);
+      }
     }
   }
 
@@ -666,6 +776,10 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
     a.n0 = n0;
     a.s1 = s1;
     a.n1 = n1;
+    a.img = tc_ok && K <= 16
+                ? append_planes(tc_img, mm_mat.data() + mm_off[l].mat, K, n1, K, K, pr.data() + s1).x
+                : -1;
+    a.plan = a.img >= 0 ? tc_plan(plan, {make_int2(K, n1), make_int2(K, n1)}, tiles, sms) : make_int2(0, 0);
   }
 
   // twiddles: tw[id][k] = psi^brev(k), itw[id][k] = psi^-brev(k)
@@ -685,6 +799,10 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
       const uint32_t e = brev(k, log_n);
       tw[(size_t)i * n + k] = shoup_pair(pw[e], q);
       itw[(size_t)i * n + k] = shoup_pair(ipw[e], q);
+    }
+    for (int k = 0; k < 64; ++k) {
+      tc_tgt[i].tw[k] = tw[(size_t)i * n + k];
+      tc_src[i].itw[k] = itw[(size_t)i * n + k];
     }
   }
 
@@ -718,10 +836,9 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
       {mm_mat.data(), mm_mat.size() * sizeof(int32_t), 0},
       {mm_epi.data(), mm_epi.size() * sizeof(MmEpi), 0},
       {tc_img.data(), tc_img.size(), 0},
-      {up_img.data(), up_img.size() * sizeof(int2), 0},
-      {dn_img.data(), dn_img.size() * sizeof(int2), 0},
-      {rs_img.data(), rs_img.size() * sizeof(int2), 0},
       {rs_qinv_r.data(), rs_qinv_r.size() * sizeof(uint2), 0},
+      {tc_src.data(), tc_src.size() * sizeof(TcSrcRec), 0},
+      {tc_tgt.data(), tc_tgt.size() * sizeof(TcTgtRec), 0},
   };
   size_t total = 0;
   for (auto& p : parts) {
@@ -738,8 +855,6 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
   ctx->d_tables = base;
   ctx->table_bytes = total;
   DevParams& dp = ctx->dp;
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || sms < 1) sms = 1;
   dp.sms = sms;
   dp.log_n = log_n;
   dp.L = L;
@@ -759,10 +874,28 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
   dp.ks.rs_mat = reinterpret_cast<const int32_t*>(base + parts[11].off);
   dp.ks.dn_pqinv = reinterpret_cast<const uint2*>(base + parts[12].off);
   dp.ks.tc_img = tc_ok ? reinterpret_cast<const uint8_t*>(base + parts[22].off) : nullptr;
-  dp.ks.up_img = reinterpret_cast<const int2*>(base + parts[23].off);
-  dp.ks.dn_img = reinterpret_cast<const int2*>(base + parts[24].off);
-  dp.ks.rs_img = reinterpret_cast<const int2*>(base + parts[25].off);
-  dp.ks.rs_qinv_r = reinterpret_cast<const uint2*>(base + parts[26].off);
+  dp.ks.rs_qinv_r = reinterpret_cast<const uint2*>(base + parts[23].off);
+  dp.ks.tc_src = reinterpret_cast<const TcSrcRec*>(base + parts[24].off);
+  dp.ks.tc_tgt = reinterpret_cast<const TcTgtRec*>(base + parts[25].off);
+  ctx->plan = std::move(plan);
+  dp.ks.h_plan = ctx->plan.data();
+  ctx->up_plan = std::move(up_plan);
+  ctx->dn_plan = std::move(dn_plan);
+  ctx->rs_plan = std::move(rs_plan);
+  dp.ks.h_up_plan = ctx->up_plan.data();
+  dp.ks.h_dn_plan = ctx->dn_plan.data();
+  dp.ks.h_rs_plan = ctx->rs_plan.data();
+  ctx->one_plan = std::move(one_plan);
+  dp.ks.h_one_plan = ctx->one_plan.data();
+  dp.ks.one_img = one_img;
+  ctx->up_off = std::move(up_off);
+  ctx->up_img = std::move(up_img);
+  ctx->dn_img = std::move(dn_img);
+  ctx->rs_img = std::move(rs_img);
+  dp.ks.h_up_off = ctx->up_off.data();
+  dp.ks.h_up_img = ctx->up_img.data();
+  dp.ks.h_dn_img = ctx->dn_img.data();
+  dp.ks.h_rs_img = ctx->rs_img.data();
   for (int l = 1; l < nlev && ctx->windowed; ++l) {
     RrArgs& r = ctx->rr[l];
     r.drop = reinterpret_cast<const int2*>(base + parts[13].off) + rr_off[l].drop;

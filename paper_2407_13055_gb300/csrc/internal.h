@@ -14,6 +14,25 @@
 
 namespace ckks {
 
+// Reduction of a tensor-core output (tc_residue in cols_tc.cuh), 32 bytes:
+// q, c = 2^16 mod q with its Shoup companion, the addends of A and B,
+// inv = floor(2^32 / q).
+struct TcPrime {
+  uint32_t q, c, csh, ea, eb, inv, pad0, pad1;
+};
+// What a tensor-core column block needs of a source's or a target's prime: the
+// column phase's 64 twiddle pairs (the tables' first entries) and the constants.
+// Consecutive primes are one bulk copy.
+struct TcSrcRec {
+  uint2 itw[64];
+  TcPrime prime;
+};
+struct TcTgtRec {
+  TcPrime prime;
+  uint2 tw[64];
+};
+constexpr int kTcMaxBlocks = 192;  // blocks of a tensor-core column kernel (one per SM)
+
 // Key-switching constants on the device (all built by host.cu).
 struct KsTables {
   // ModUp (Alg. 1 Q_j -> PQ): for the level with n ciphertext limbs and digit
@@ -48,12 +67,26 @@ struct KsTables {
   // conversion matrices in the shared-memory layout of the MMA's B operand,
   // one allocation tc_img; entries (byte offset, bytes) per conversion:
   // up_img[tix * dnum + j] (ModUp digit j), dn_img[tix] (ModDown),
-  // rs_img[n] (fused ModDown + rescale at n limbs). Null tc_img: the
-  // tensor-core kernels are not available (more than 16 sources).
+  // rs_img[n] (fused ModDown + rescale at n limbs), all h_*; MmArgs::img. Null tc_img:
+  // the tensor-core kernels are not available (more than 16 sources).
+  // tc_src, tc_tgt: per prime, its column twiddles and reduction constants.
   const uint8_t* tc_img;
-  const int2* up_img;
-  const int2* dn_img;
-  const int2* rs_img;
+  const TcSrcRec* tc_src;
+  const TcTgtRec* tc_tgt;
+  // Host copies (the context's) of the offsets, for the launchers.
+  const int2* h_up_off;
+  const int2* h_up_img;
+  const int2* h_dn_img;
+  const int2* h_rs_img;
+  int one_img;  // offset of the one-source image [1]_{q_i}, i < L - 1 (rescaling by one prime)
+  // Division of the tensor-core column kernels' work: block boundaries in
+  // h_plan (host) at (offset, blocks) per conversion (h_up_plan[tix],
+  // h_dn_plan[tix], h_rs_plan[n], h_one_plan[n], MmArgs::plan, RrArgs::plan).
+  const uint32_t* h_plan;
+  const int2* h_up_plan;
+  const int2* h_dn_plan;
+  const int2* h_rs_plan;
+  const int2* h_one_plan;
 };
 
 struct DevParams {
@@ -64,7 +97,6 @@ struct DevParams {
   KsTables ks;
   int sms = 0;  // streaming multiprocessors of the context's device (grid sizing)
   int pdl;  // host-side launch option: key-switch kernels use programmatic dependent launch
-  int tune_tensor = 0;  // host-side option: the fine-tuner also times the tensor-core column shapes
   int unfused = 0;      // host-side option: key-switching operations run the unfused one-step-per-launch form
   int checked = 0;      // host-side option: range checks of operands and results (CKKS_LAUNCH_CHECKED)
   int rows_passes = 3;  // host-side launch option at N = 2^16: row phase in 3 (16 values per
@@ -171,6 +203,8 @@ struct MmArgs {
                        //      dropped prime (its row source is Y P^-1), 1 for p_k
   const int32_t* mat;  // [n1][K]: [(P T_drop / s_k) 2^32]_t, centered
   const MmEpi* epi;    // [n1]
+  int img;             // byte offset of the matrix's plane image, -1 above 16 sources
+  int2 plan;           // its work division in h_plan
 };
 
 struct RrArgs {
@@ -181,6 +215,8 @@ struct RrArgs {
   const uint2* cin;
   const int32_t* mat;
   const RrEpi* epi;
+  int img;    // as in MmArgs
+  int2 plan;
 };
 
 // Kernel ids of the key-switch and rescale pipelines (measurement support).
@@ -363,7 +399,9 @@ void launch_rational_rescale(const DevParams& dp, const Scratch& sc, const RrArg
 void launch_moddown(const DevParams& dp, const Scratch& sc, const uint32_t* acc, int n, uint32_t* out,
                     cudaStream_t st);
 // Rescale: in [2][n][N] (stride sin) -> out [2][n-1][N] (stride sout).
-void launch_rescale(const DevParams& dp, const Scratch& sc, const uint32_t* in, size_t sin, int n,
+// tensor: the column phase may run in its tensor-core form, whose first launch
+// sets a kernel attribute (ckks_rescale_noalloc passes false).
+void launch_rescale(const DevParams& dp, bool tensor, const Scratch& sc, const uint32_t* in, size_t sin, int n,
                     uint32_t* out, size_t sout, cudaStream_t st);
 
 // ---- launchers (k_bconv.cu) ----
@@ -427,6 +465,8 @@ struct ckks_ctx {
   std::vector<int> lvl_first, lvl_count;
   std::vector<int> rows_off, rows_cnt;  // per level + 1: ModUp row-table range
   std::vector<ckks::RrArgs> rr;         // per level l >= 1 (windowed): transition l -> l - 1
+  std::vector<uint32_t> plan;
+  std::vector<int2> up_off, up_img, dn_img, rs_img, up_plan, dn_plan, rs_plan, one_plan;  // host copies behind dp.ks.h_* (the parent's, for a clone)
   std::vector<ckks::MmArgs> mm;         // per level l >= 1: merged ModDown + rescaling l -> l - 1
   int n_levels() const { return (int)lvl_count.size(); }
   int lvl_n(int level) const { return lvl_count[level]; }

@@ -1,0 +1,13 @@
+// Tensor-core column kernels (N = 2^16 and 2^12; the smallest ring has none).
+#include "cols.cuh"
+
+namespace ckks {
+
+template void launch_cols_tc<Geo<8, 32>, false>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
+template void launch_cols_tc<Geo<8, 32>, true>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
+template void launch_cols_tc<Geo<8, 8>, false>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
+template void launch_cols_tc<Geo<8, 8>, true>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
+template void launch_cols_tc<Geo<4, 4>, false>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
+template void launch_cols_tc<Geo<4, 4>, true>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
+
+}  // namespace ckks

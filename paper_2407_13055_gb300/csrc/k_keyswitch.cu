@@ -687,6 +687,16 @@ static void stream_grid(int log_n, int limbs, dim3& grid, int& threads) {
 // window [base, base + n).
 static int active_digits(const KsArgs& a, int alpha) { return (a.base + a.n - 1) / alpha - a.base / alpha + 1; }
 
+// BConv products per coefficient of the level's ModUp.
+static int modup_work(const KsArgs& a, int alpha) {
+  int w = 0;
+  for (int j = a.base / alpha; j <= (a.base + a.n - 1) / alpha; ++j) {
+    const int k = std::min(a.n, (j + 1) * alpha - a.base) - std::max(0, j * alpha - a.base);
+    w += k * (a.n + alpha - k);
+  }
+  return w;
+}
+
 // Row map of the level's n ciphertext limbs (window primes).
 static LimbMap window_map(const KsArgs& a, int L) {
   LimbMap m{nullptr, 0, a.n, a.n, L};
@@ -706,7 +716,7 @@ static void moddown_rescale_tail(const DevParams& dp, const Scratch& sc, const K
   in_map.tail_prime = top;
   launch_rows_inv<G>(dp, SrcModDownTop{a, A, a_stride}, sc.S, 2 * alpha + 2, in_map, true, st);
   prof_mark(sc, st, P_MODDOWN_IN_ROWS);
-  launch_rs_cols_fused<G>(dp, n, sc, T3, pick_shape<G>(sc, CK_RS_FUSED, a.tix, default_shape<G>(2, dp.sms)), st);
+  launch_rs_cols_fused<G>(dp, n, sc, T3, pick_shape<G>(sc, CK_RS_FUSED, a.tix, alpha + 1, 2 * (alpha + 1) * top), st);
   prof_mark(sc, st, P_RS_COLS);
   launch_rows_fwd<G>(dp, T3, EpiRsOut{a, A, a_stride}, 2 * top, LimbMap{nullptr, 0, top, top, dp.L}, st);
   prof_mark(sc, st, P_RS_ROWS);
@@ -722,7 +732,7 @@ static void merged_tail(const DevParams& dp, const Scratch& sc, const KsArgs& a,
   const int ext = a.n + dp.alpha;
   launch_rows_inv<G>(dp, SrcMerged{a, A, ext}, sc.S, 2 * m.K, LimbMap{m.rows, 0, 0, 0, 0}, true, st);
   prof_mark(sc, st, P_MODDOWN_IN_ROWS);
-  launch_mm_cols<G>(dp, m, sc, pick_shape<G>(sc, CK_RS_FUSED, a.tix, default_shape<G>(2, dp.sms)), st);
+  launch_mm_cols<G>(dp, m, sc, pick_shape<G>(sc, CK_RS_FUSED, a.tix, m.K, 2 * m.K * m.n1), st);
   prof_mark(sc, st, P_RS_COLS);
   LimbMap out_map{nullptr, 0, m.n1, m.n1, dp.L};
   out_map.base = m.s1;
@@ -739,7 +749,7 @@ static void moddown_tail(const DevParams& dp, const Scratch& sc, const KsArgs& a
   launch_rows_g<G>(dp, true, A, sc.S, 2 * alpha,
                    LimbMap{nullptr, n, n + alpha, n, dp.L, alpha, (int)(a_stride >> dp.log_n)}, true, st);
   prof_mark(sc, st, P_MODDOWN_IN_ROWS);
-  launch_moddown_cols<G>(dp, n, a.base, a.tix, sc, pick_shape<G>(sc, CK_MODDOWN, a.tix, default_shape<G>(2, dp.sms)), st);
+  launch_moddown_cols<G>(dp, n, a.base, a.tix, sc, pick_shape<G>(sc, CK_MODDOWN, a.tix, alpha, 2 * alpha * n), st);
   prof_mark(sc, st, P_MODDOWN_COLS);
   launch_rows_fwd<G>(dp, sc.T, EpiModDown{a, A, a_stride}, 2 * n, window_map(a, dp.L), st);
   prof_mark(sc, st, P_MODDOWN_ROWS);
@@ -767,7 +777,7 @@ void launch_ks_modup(const DevParams& dp0, const Scratch& sc, const KsArgs& a, c
     launch_rows_inv<G>(dp, SrcKsInput{a}, sc.S, a.n, window_map(a, dp.L), true, st);
     prof_mark(sc, st, P_KS_IN_ROWS);
     launch_modup_cols<G>(dp, a.n, a.base, a.tix, digits, sc,
-                         pick_shape<G>(sc, CK_MODUP, a.tix, default_shape<G>(digits, dp.sms)), st);
+                         pick_shape<G>(sc, CK_MODUP, a.tix, dp.alpha, modup_work(a, dp.alpha)), st);
     prof_mark(sc, st, P_MODUP_COLS);
     launch_rows_g<G>(dp, false, sc.T, sc.T, a.rows_cnt, LimbMap{dp.ks.up_rows + a.rows_off, 0, 1, 0, 0}, false, st);
     prof_mark(sc, st, P_MODUP_ROWS);
@@ -936,13 +946,7 @@ void launch_persistent(const DevParams& dp, const PersOp* ops, const int2* items
 template <class G>
 static std::vector<ColShape> shape_candidates(int targets, const ColShape& def, bool tensor) {
   std::vector<ColShape> v;
-  if (tensor)
-    for (int tc : {8, 4})
-      for (int sl : {2, 4, 8})
-        for (int nc : {8, 16}) {
-          const ColShape c{tc, sl, 1, nc};
-          if (tc_shape_ok<G>(c)) v.push_back(c);
-        }
+  if (tensor) v.push_back(ColShape{8, 4, 1, 16});  // the tensor-core shapes all run one kernel
   for (int tc : {8, 4}) {
     if (G::W % tc != 0) continue;
     for (int sl : {2, 4, 8})
@@ -976,18 +980,18 @@ int tune_columns(const DevParams& dp, const Scratch& sc, Tuning& tu, const KsArg
       ColShape def;
       int targets;
       const bool tensor =
-          dp.tune_tensor && dp.ks.tc_img != nullptr && dp.alpha + (k == CK_RS_FUSED ? 1 : 0) <= kTcMaxSources;
+          G::H == 64 && dp.ks.tc_img != nullptr && dp.alpha + (k == CK_RS_FUSED ? 1 : 0) <= kTcMaxSources;
       std::function<void(const ColShape&)> run;
       if (k == CK_MODUP) {
-        def = default_shape<G>(digits, dp.sms);
+        def = default_shape<G>(CK_MODUP, alpha);
         targets = n;  // fewest targets of a digit: n + alpha - (digit size)
         run = [&](const ColShape& s) { launch_modup_cols<G>(dp, n, base, tix, digits, sc, s, st); };
       } else if (k == CK_MODDOWN) {
-        def = default_shape<G>(2, dp.sms);
+        def = default_shape<G>(CK_MODDOWN, alpha);
         targets = n;
         run = [&](const ColShape& s) { launch_moddown_cols<G>(dp, n, base, tix, sc, s, st); };
       } else {
-        def = default_shape<G>(2, dp.sms);
+        def = default_shape<G>(CK_RS_FUSED, alpha + 1);
         targets = n - 1;
         run = [&](const ColShape& s) {
           launch_rs_cols_fused<G>(dp, n, sc, sc.T, s, st);
@@ -1073,7 +1077,7 @@ void launch_hoisted_rotations(const DevParams& dp0, const Scratch& sc, const KsA
     launch_rows_g<G>(dp, true, a0.x0 + a0.poly_stride0, sc.S, n, window_map(a0, dp.L), true, st);
     prof_mark(sc, st, P_KS_IN_ROWS);
     launch_modup_cols<G>(dp, n, a0.base, a0.tix, digits, sc,
-                         pick_shape<G>(sc, CK_MODUP, a0.tix, default_shape<G>(digits, dp.sms)), st);
+                         pick_shape<G>(sc, CK_MODUP, a0.tix, dp.alpha, modup_work(a0, dp.alpha)), st);
     prof_mark(sc, st, P_MODUP_COLS);
     launch_rows_g<G>(dp, false, sc.T, sc.T, a0.rows_cnt, LimbMap{dp.ks.up_rows + a0.rows_off, 0, 1, 0, 0}, false,
                      st);
@@ -1108,7 +1112,7 @@ void launch_linear_transform(const DevParams& dp0, const Scratch& sc, const KsAr
       launch_rows_g<G>(dp, true, a.x0 + a.poly_stride0, sc.S, n, window_map(a, dp.L), true, st);
       prof_mark(sc, st, P_KS_IN_ROWS);
       launch_modup_cols<G>(dp, n, a.base, a.tix, digits, sc,
-                           pick_shape<G>(sc, CK_MODUP, a.tix, default_shape<G>(digits, dp.sms)), st);
+                           pick_shape<G>(sc, CK_MODUP, a.tix, dp.alpha, modup_work(a, dp.alpha)), st);
       prof_mark(sc, st, P_MODUP_COLS);
       launch_rows_g<G>(dp, false, sc.T, sc.T, a.rows_cnt, LimbMap{dp.ks.up_rows + a.rows_off, 0, 1, 0, 0}, false,
                        st);
@@ -1121,7 +1125,7 @@ void launch_linear_transform(const DevParams& dp0, const Scratch& sc, const KsAr
       launch_rows_g<G>(dp, true, sc.A, down.S, 2 * alpha,
                        LimbMap{nullptr, n, n + alpha, n, dp.L, alpha, (int)(a_stride >> dp.log_n)}, true, st);
       prof_mark(sc, st, P_MODDOWN_IN_ROWS);
-      launch_moddown_cols<G>(dp, n, a.base, a.tix, down, pick_shape<G>(sc, CK_MODDOWN, a.tix, default_shape<G>(2, dp.sms)), st);
+      launch_moddown_cols<G>(dp, n, a.base, a.tix, down, pick_shape<G>(sc, CK_MODDOWN, a.tix, alpha, 2 * alpha * n), st);
       prof_mark(sc, st, P_MODDOWN_COLS);
       launch_rows_g<G>(dp, false, down.T, down.T, 2 * n, window_map(a, dp.L), false, st);
       prof_mark(sc, st, P_MODDOWN_ROWS);
@@ -1170,7 +1174,7 @@ void launch_moddown(const DevParams& dp, const Scratch& sc, const uint32_t* acc,
   });
 }
 
-void launch_rescale(const DevParams& dp, const Scratch& sc, const uint32_t* in, size_t sin, int n,
+void launch_rescale(const DevParams& dp, bool tensor, const Scratch& sc, const uint32_t* in, size_t sin, int n,
                     uint32_t* out, size_t sout, cudaStream_t st) {
   const int top = n - 1;
   if (top < 1) return;
@@ -1179,10 +1183,17 @@ void launch_rescale(const DevParams& dp, const Scratch& sc, const uint32_t* in, 
     // top limb of both polynomials -> S [2] (compact)
     launch_rows_g<G>(dp, true, in, sc.S, 2, LimbMap{nullptr, top, n, n, dp.L, 1, (int)(sin >> dp.log_n)}, true, st);
     prof_mark(sc, st, P_RS_IN_ROWS);
-    const int tiles = G::W / G::TC;
-    const int gr = groups_for(tiles * 2, top, dp.sms);
-    launch_pdl(dp.pdl, k_rs_cols<G>, dim3(tiles, 2, gr), dim3(G::CT), 0, st, dp, n, (const uint32_t*)sc.S, sc.T, gr);
-    count_launch(1);
+    // tensor-core form from 12 targets on (product, sum and rescale at level 13
+    // 31.0 us in either form, 30 53.4 against 60.4, 39 63.7 against 73.8, below
+    // it the start of its blocks shows: level 4 22.7 against 20.6)
+    if (tensor && G::W == 1024 && dp.ks.tc_img && top >= 12) {
+      launch_rescale_tc<G>(dp, n, sc, st);
+    } else {
+      const int tiles = G::W / G::TC;
+      const int gr = groups_for(tiles * 2, top, dp.sms);
+      launch_pdl(dp.pdl, k_rs_cols<G>, dim3(tiles, 2, gr), dim3(G::CT), 0, st, dp, n, (const uint32_t*)sc.S, sc.T, gr);
+      count_launch(1);
+    }
     prof_mark(sc, st, P_RS_COLS);
     launch_rows_fwd<G>(dp, sc.T, EpiRescale{in, sin, top, out, sout}, 2 * top, LimbMap{nullptr, 0, top, top, dp.L},
                        st);

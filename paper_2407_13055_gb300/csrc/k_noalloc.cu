@@ -80,7 +80,7 @@ extern "C" int ckks_rescale_noalloc(ckks_ctx* ctx, const uint32_t* in_dev, int l
   sc.S = base;
   sc.T = base + 2 * limb;
   const int n = level + 1;
-  ckks::launch_rescale(ctx->dp, sc, in_dev, (size_t)n * limb, n, out_dev, (size_t)level * limb, ctx->stream);
+  ckks::launch_rescale(ctx->dp, false, sc, in_dev, (size_t)n * limb, n, out_dev, (size_t)level * limb, ctx->stream);
   const cudaError_t le = cudaGetLastError();
   if (le != cudaSuccess) {
     ctx->err = std::string("rescale_noalloc: ") + cudaGetErrorString(le);

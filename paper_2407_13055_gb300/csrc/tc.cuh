@@ -9,11 +9,10 @@
 // each m' is split the same way into four bytes e_(k,a,b) ("planes" b). Every
 // byte is an exact fp16 value and every product d e (|d e| <= 2^14) an exact
 // fp32 value, and plane b's sum over the K sources and 4 digits,
-// P_b = sum_(k,a) d_(k,a) e_(k,a,b), stays below 2^22 in magnitude for
-// K <= 63, so the fp32 accumulation is exact in any order. Then
-// S = sum_b P_b 2^(8b) = sum_k y_k m_k + (multiple of p), |S| < 2^46, and one
-// signed Montgomery reduction (Alg. 2) gives the same residue as the
-// CUDA-core lazy sum.
+// P_b = sum_(k,a) d_(k,a) e_(k,a,b), stays below 2^20 in magnitude for
+// K <= 16 (448 2^7 per source), so the fp32 accumulation is exact in any order.
+// Then sum_b P_b 2^(8b) = sum_k y_k m_k modulo p; reduced, it is the residue
+// that the CUDA-core lazy sum gives.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -44,20 +43,28 @@ __host__ __device__ constexpr uint32_t idesc_f16(int m, int n) {
   return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// D[tmem] (+)= A * B^T, issued by one thread; completion is tracked with
-// commit().
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, int accumulate) {
+// D[tmem] (+)= A[tmem] * B^T, executed by a whole converged warp and issued by
+// one elected lane; completion is tracked with commit(). A: one tensor-memory
+// lane per row, two consecutive K elements per 32-bit column. The election
+// sits in the instruction's predicate: under a branch on the lane the operands
+// cannot be uniform registers, and an issue took 119 cycles instead of 8
+// (32 products of N = 16: 3946 against 408 cycles to their completion).
+template <bool ACCUMULATE>
+__device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc) {
   asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+      "{\n.reg .pred p, q;\nelect.sync _|q, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b), "r"(idesc), "n"(ACCUMULATE ? 1 : 0)
+      : "memory");
 }
 
 // The mbarrier at mbar receives one arrival when every tcgen05.mma issued so
-// far by this thread has completed.
+// far by the elected lane of this (whole, converged) warp has completed.
 __device__ __forceinline__ void commit(uint32_t mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-               : "memory");
+  asm volatile(
+      "{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\n"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(mbar)
+      : "memory");
 }
 
 // Tensor-memory allocation: executed by one whole warp; the base address is
@@ -73,17 +80,31 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// 16 consecutive fp32 columns of this thread's TMEM lane (the warp reads the
-// 32 lanes of its quadrant, warp id mod 4); taddr carries the quadrant's
-// first lane in its upper half.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
+// Four consecutive 32-bit columns of this thread's TMEM lane (the warp reads
+// the 32 lanes of its quadrant, warp id mod 4); taddr carries the quadrant's
+// first lane in its upper half. And two columns written.
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t& a, uint32_t& b, uint32_t& c, uint32_t& d) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(a), "=r"(b), "=r"(c), "=r"(d)
+               : "r"(taddr)
+               : "memory");
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Waits for this thread's loads; the registers pass through the statement so
+// that nothing reads them before it.
+__device__ __forceinline__ void tmem_wait_ld32(uint32_t (&f)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(f[0]), "+r"(f[1]), "+r"(f[2]), "+r"(f[3]), "+r"(f[4]), "+r"(f[5]), "+r"(f[6]), "+r"(f[7]),
+                 "+r"(f[8]), "+r"(f[9]), "+r"(f[10]), "+r"(f[11]), "+r"(f[12]), "+r"(f[13]), "+r"(f[14]), "+r"(f[15]),
+                 "+r"(f[16]), "+r"(f[17]), "+r"(f[18]), "+r"(f[19]), "+r"(f[20]), "+r"(f[21]), "+r"(f[22]),
+                 "+r"(f[23]), "+r"(f[24]), "+r"(f[25]), "+r"(f[26]), "+r"(f[27])
+               :
+               : "memory");
+  asm volatile("" : "+r"(f[28]), "+r"(f[29]), "+r"(f[30]), "+r"(f[31])::"memory");
+}
+__device__ __forceinline__ void tmem_st2(uint32_t taddr, uint32_t a, uint32_t b) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};" ::"r"(taddr), "r"(a), "r"(b) : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Generic-proxy shared-memory writes become visible to the async proxy
 // (tensor core, bulk copies).
@@ -133,6 +154,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long l
   return false;
 }
 
+__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
+}
+
 // One arrival that also expects `bytes` of transaction (bulk-copy) data.
 __device__ __forceinline__ void mbar_expect_tx(uint32_t mbar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
@@ -158,38 +183,17 @@ __device__ __forceinline__ void report_timeout(uint32_t* status) {
   if (status) atomicOr(status, kStatusTimeout);
 }
 
-// Four balanced signed-byte digits of a centered residue (|y| < 2^30) as two
-// fp16 pairs, in order d0 d1 | d2 d3: with z = y + 0x808080 the low three
-// bytes of z are d_a + 128 (a < 3) and z >> 24 = d3 in [-64, 64]. Each byte u
-// becomes the fp16 1024 + u by placing 0x64 above it; subtracting 1152 then
-// leaves u - 128 exactly.
-__device__ __forceinline__ uint2 digits_f16(int32_t y) {
-  const uint32_t z = (uint32_t)(y + 0x808080);
+// Four balanced signed-byte digits of a centered residue y (|y| < 2^30) as two
+// fp16 pairs, in order d0 d1 | d2 d3, from z = y + 0x80808080: byte a of z is
+// d_a + 128 (d3 in [-64, 64]). Each byte u becomes the fp16 1024 + u by placing
+// 0x64 above it; subtracting 1152 then leaves u - 128 exactly.
+__device__ __forceinline__ uint2 digits_f16(uint32_t z) {
   uint32_t lo = __byte_perm(z, 0x64646464u, 0x4140);
-  uint32_t hi = __byte_perm(z, 0x64646464u, 0x4342) ^ 0x00800000u;
+  uint32_t hi = __byte_perm(z, 0x64646464u, 0x4342);
   const __half2 off = __halves2half2(__ushort_as_half((unsigned short)0x6480), __ushort_as_half((unsigned short)0x6480));
   __half2 a = __hsub2(*reinterpret_cast<__half2*>(&lo), off);
   __half2 b = __hsub2(*reinterpret_cast<__half2*>(&hi), off);
   return make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
-}
-
-// Residue in [0, p) of an output from its four plane sums (fp32 bit patterns
-// of exact integers with |v| < 2^22): adding 1.5 2^23 puts v + 0x4B400000 in
-// the float's bit pattern; S = sum_b v_b 2^(8b) is assembled from two 32-bit
-// halves t0 = v0 + 2^8 v1, t1 = v2 + 2^8 v3 (each fits int32), then
-// S 2^-32 mod p by SMR (the matrix carries the 2^32).
-__device__ __forceinline__ uint32_t planes_residue(uint32_t f0, uint32_t f1, uint32_t f2, uint32_t f3, uint32_t p,
-                                                   uint32_t m) {
-  const float kMagic = 12582912.0f;
-  const uint32_t b0 = __float_as_uint(__fadd_rn(__uint_as_float(f0), kMagic));
-  const uint32_t b1 = __float_as_uint(__fadd_rn(__uint_as_float(f1), kMagic));
-  const uint32_t b2 = __float_as_uint(__fadd_rn(__uint_as_float(f2), kMagic));
-  const uint32_t b3 = __float_as_uint(__fadd_rn(__uint_as_float(f3), kMagic));
-  constexpr uint32_t kBias = 0x4B400000u * 257u;  // (1 + 2^8) times the magic's pattern, mod 2^32
-  const int32_t t0 = (int32_t)(b0 + (b1 << 8) - kBias);
-  const int32_t t1 = (int32_t)(b2 + (b3 << 8) - kBias);
-  const int64_t S = (int64_t)t0 + ((int64_t)t1 << 16);
-  return fix_signed(smr(S, p, m), p);
 }
 
 }  // namespace tc
