@@ -20,6 +20,14 @@ struct PrimeConst {
 // a in [0, 2b) -> [0, b): min(a, a - b) on unsigned values.
 __device__ __forceinline__ uint32_t csub(uint32_t a, uint32_t b) { return min(a, a - b); }
 
+// 2q for q < 2^31 as a rotation. Written as a product or a shift, the compiler
+// folds it into every a - 2q (a multiply-add), which keeps that subtraction
+// from joining the minimum of csub in one instruction and the three-operand
+// sums of the butterflies from being one: 8 instructions per lazy butterfly
+// instead of 6 (N = 2^16, dnum = 3, top level: HRot 139.3 -> 133.3 us, HMult +
+// rescale 158.1 -> 153.1).
+__device__ __forceinline__ uint32_t twice(uint32_t q) { return __funnelshift_l(q, q, 1); }
+
 // Signed Montgomery reduction (Alg. 2): for x in [-q 2^31, q 2^31),
 // y = x 2^-32 mod q with y in (-q, q): one low and one high signed product.
 __device__ __forceinline__ int32_t smr(int64_t x, uint32_t q, uint32_t m) {
@@ -75,7 +83,7 @@ __device__ __forceinline__ uint32_t fix_signed(int32_t v, uint32_t q) {
 template <bool LAZY>
 __device__ __forceinline__ void ct_bfly(uint32_t& x, uint32_t& y, uint32_t w, uint32_t wsh, uint32_t q) {
   if (LAZY) {
-    const uint32_t q2 = 2 * q;
+    const uint32_t q2 = twice(q);
     x = csub(x, q2);
     uint32_t t = shoup(y, w, wsh, q);
     y = x - t + q2;
@@ -91,7 +99,7 @@ __device__ __forceinline__ void ct_bfly(uint32_t& x, uint32_t& y, uint32_t w, ui
 template <bool LAZY>
 __device__ __forceinline__ void gs_bfly(uint32_t& x, uint32_t& y, uint32_t w, uint32_t wsh, uint32_t q) {
   if (LAZY) {
-    const uint32_t q2 = 2 * q;
+    const uint32_t q2 = twice(q);
     uint32_t s = x + y;
     uint32_t d = x - y + q2;
     x = csub(s, q2);
@@ -109,7 +117,7 @@ __device__ __forceinline__ void gs_bfly(uint32_t& x, uint32_t& y, uint32_t w, ui
 // Reduce a lazily reduced value to [0, q).
 template <bool LAZY>
 __device__ __forceinline__ uint32_t normalize(uint32_t x, uint32_t q) {
-  if (LAZY) x = csub(x, 2 * q);
+  if (LAZY) x = csub(x, twice(q));
   return csub(x, q);
 }
 
