@@ -472,7 +472,7 @@ int ckks_rescale_noalloc(ckks_ctx* ctx, const uint32_t* in_dev, int level, uint3
 #define CKKS_LAUNCH_CHECKED 8
 int ckks_set_launch_flags(ckks_ctx* ctx, int flags);
 
-/* Bounded device-side waits. The tensor-core and bulk-copy kernels wait on
+/* Bounded device-side waits. The tensor-core column kernels wait on
  * shared-memory barriers (for their bulk copies and matrix products); each
  * wait gives up after `cycles` SM clock cycles (default 2^32, about two
  * seconds), marks the context's status word, frees what the block holds and
@@ -511,16 +511,8 @@ int ckks_set_wait_limit(ckks_ctx* ctx, long long cycles);
  * register passes (32 values per thread, radix 2^5 x 2^5) or 3 (16 values,
  * 2^4 x 2^3 x 2^3); the entry's tc is the number of passes (sl = z = tp = 1),
  * tuned on the level's ModUp NTT rows and used by that level's key
- * switches. tc = 4 and 5 select the three-pass form whose forward rows take
- * 2 (4) and 4 (5) row pairs per block and stage each pair's input in shared
- * memory with bulk copies (cp.async.bulk) that overlap the previous pair's
- * arithmetic (bounded waits, see ckks_set_wait_limit). tc = 6 selects the
- * three-pass form with the second and third passes' twiddles copied into
- * shared memory by asynchronous copies (cp.async) instead of held in
- * registers (64 registers, 8 blocks of 4 warps per SM), forward and inverse
- * rows; ckks_tune does not time it (slower than form 3 on GB300, most of all
- * for the rows with fused epilogues), it is set by hand only. Without an
- * entry: 3. */
+ * switches. tc = 4, 5 and 6 are accepted and select the three-pass kernels,
+ * too. Without an entry: 3. */
 #define CKKS_ROW_PASSES 3
 /* Times every candidate shape of the three kernels at `level` (reps launches
  * each, CUDA events on the context stream, on the context's scratch), and at

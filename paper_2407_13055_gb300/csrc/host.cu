@@ -806,6 +806,31 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
     }
   }
 
+  // N = 2^16: twiddles of the last three row stages in the three-pass row
+  // kernels' order: row h, unit k, thread t. Stage s of group g's block b is
+  // entry (64 + h) 128 2^s + (2 t + g) 2^s + b.
+  std::vector<uint2> twc, itwc;
+  if (log_n == 16) {
+    twc.resize((size_t)np * 64 * 7 * 64 * 2);
+    itwc.resize(twc.size());
+    for (int dir = 0; dir < 2; ++dir) {
+      const uint2* from = dir ? itw.data() : tw.data();
+      uint2* to = dir ? itwc.data() : twc.data();
+      for (int i = 0; i < np; ++i)
+        for (int h = 0; h < 64; ++h) {
+          const uint2* t0 = from + (size_t)i * n;
+          uint2* u = to + ((size_t)i * 64 + h) * 7 * 128;
+          const int base = (64 + h) * 128;
+          for (int t = 0; t < 64; ++t)
+            for (int e = 0; e < 2; ++e) {
+              u[2 * t + e] = t0[base + 2 * t + e];
+              for (int k = 0; k < 2; ++k) u[(1 + k) * 128 + 2 * t + e] = t0[2 * base + 4 * t + 2 * k + e];
+              for (int k = 0; k < 4; ++k) u[(3 + k) * 128 + 2 * t + e] = t0[4 * base + 8 * t + 2 * k + e];
+            }
+        }
+    }
+  }
+
   // one device allocation for all tables
   struct Part {
     const void* src;
@@ -839,6 +864,8 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
       {rs_qinv_r.data(), rs_qinv_r.size() * sizeof(uint2), 0},
       {tc_src.data(), tc_src.size() * sizeof(TcSrcRec), 0},
       {tc_tgt.data(), tc_tgt.size() * sizeof(TcTgtRec), 0},
+      {twc.data(), twc.size() * sizeof(uint2), 0},
+      {itwc.data(), itwc.size() * sizeof(uint2), 0},
   };
   size_t total = 0;
   for (auto& p : parts) {
@@ -863,6 +890,8 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
   dp.pc = reinterpret_cast<const PrimeConst*>(base + parts[0].off);
   dp.tw = reinterpret_cast<const uint2*>(base + parts[1].off);
   dp.itw = reinterpret_cast<const uint2*>(base + parts[2].off);
+  dp.twc = reinterpret_cast<const uint4*>(base + parts[26].off);
+  dp.itwc = reinterpret_cast<const uint4*>(base + parts[27].off);
   dp.ks.up_cin = reinterpret_cast<const uint2*>(base + parts[3].off);
   dp.ks.up_mat = reinterpret_cast<const int32_t*>(base + parts[4].off);
   dp.ks.up_off = reinterpret_cast<const int2*>(base + parts[5].off);

@@ -94,6 +94,10 @@ struct DevParams {
   const PrimeConst* pc;  // [L + alpha]
   const uint2* tw;       // [L + alpha][N] forward twiddles (w, Shoup companion)
   const uint2* itw;      // [L + alpha][N] inverse twiddles
+  // N = 2^16: the last three row stages' twiddles in the order the three-pass
+  // row kernels read them (rows.cuh), [L + alpha][64 rows][7][64] 16-byte units
+  const uint4* twc = nullptr;
+  const uint4* itwc = nullptr;
   KsTables ks;
   int sms = 0;  // streaming multiprocessors of the context's device (grid sizing)
   int pdl;  // host-side launch option: key-switch kernels use programmatic dependent launch
@@ -101,8 +105,8 @@ struct DevParams {
   int checked = 0;      // host-side option: range checks of operands and results (CKKS_LAUNCH_CHECKED)
   int rows_passes = 3;  // host-side launch option at N = 2^16: row phase in 3 (16 values per
                         // thread, 64 threads per row) or 2 (32 values, 32 threads) passes
-  // Bounded device-side waits (mbarrier waits of the tensor-core and bulk-copy
-  // kernels): a wait gives up after wait_limit SM clock cycles and sets
+  // Bounded device-side waits (mbarrier waits of the tensor-core kernels,
+  // admission waits of the persistent batch): a wait gives up after wait_limit SM clock cycles and sets
   // tc::kStatusTimeout in *status (host-mapped memory of the context, read
   // back by the synchronizing calls as CKKS_ETIMEOUT).
   uint32_t* status = nullptr;

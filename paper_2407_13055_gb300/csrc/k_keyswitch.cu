@@ -328,54 +328,77 @@ __global__ void k_lt_epilogue(DevParams dp, KsArgs a, LtArgs lt, const uint32_t*
   store_vec<4>(a.out + u * a.out_stride + off, z);
 }
 
-// Extra term of the ModDown output at limb i (HMult: d0 or d1; HRot: phi(b)).
-__device__ __forceinline__ void ks_extra4(const DevParams& dp, const KsArgs& a, int u, int i, uint32_t p0,
-                                          const PrimeConst& P, uint32_t (&e)[4]) {
-  const size_t off = ((size_t)i << dp.log_n) + p0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) e[k] = 0;
-  if (a.extra == 1) {
-    uint32_t b1[4], b2[4];
-    load_vec<4>(b1, a.x0 + off);
-    load_vec<4>(b2, a.x1 + off);
-    if (u == 0) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) e[k] = mulmod(b1[k], b2[k], P);
-    } else {
-      uint32_t a1[4], a2[4];
-      load_vec<4>(a1, a.x0 + a.poly_stride0 + off);
-      load_vec<4>(a2, a.x1 + a.poly_stride1 + off);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) e[k] = addm(mulmod(a1[k], b2[k], P), mulmod(a2[k], b1[k], P), P.q);
-    }
-  } else if (a.extra == 2 && u == 0) {
-    const uint32_t* sb = a.x0 + ((size_t)i << dp.log_n);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) e[k] = __ldg(sb + auto_src(p0 + k, a.galois, dp.log_n));
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Row-kernel sources and epilogues (the streaming steps fused into the row
-// phases): a thread handles positions pos0 .. pos0 + E - 1 of launch limb y,
-// four at a time.
+// phases): a thread handles E / 4 runs of four positions of launch limb y, run
+// c at pos0 + CS c.
 // ---------------------------------------------------------------------------
 
 // Key-switch input before the iNTT rows: d, a1 a2 or phi_k(a) at limb y.
 struct SrcKsInput {
   KsArgs a;
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int y, int2,
-                                             uint32_t pos0) const {
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], int y, int2, uint32_t pos0) const {
+    const size_t limb = (size_t)y << dp.log_n;
+    if (a.mode == KS_PLAIN) {
+      load_runs<E, CS>(x, a.x0 + limb + pos0);
+    } else if (a.mode == KS_TENSOR) {
+      const PrimeConst P = dp.pc[a.base + y];
+      uint32_t a2[E];
+      load_runs<E, CS>(x, a.x0 + a.poly_stride0 + limb + pos0);
+      load_runs<E, CS>(a2, a.x1 + a.poly_stride1 + limb + pos0);
 #pragma unroll
-    for (int c = 0; c < E / 4; ++c) {
-      uint32_t v[4];
-      ks_input4(dp, a, y, pos0 + 4 * c, v);
+      for (int k = 0; k < E; ++k) x[k] = mulmod(x[k], a2[k], P);
+    } else {
+      const uint32_t* s = a.x0 + a.poly_stride0 + limb;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) x[4 * c + k] = v[k];
+      for (int k = 0; k < E; ++k) x[k] = __ldg(s + auto_src(pos0 + CS * (k / 4) + k % 4, a.galois, dp.log_n));
     }
   }
 };
+
+// Extra term of the ModDown output at limb i for E positions (HMult: d0 or d1;
+// HRot: phi(b)), in halves whose loads are issued together. MONT: HMult's d0 /
+// d1 times 2^-32 (one Montgomery reduction; the caller's constant carries the
+// 2^32 back).
+template <int E, int CS, bool MONT>
+__device__ __forceinline__ void ks_extra_runs(const DevParams& dp, const KsArgs& a, int u, int i, uint32_t pos0,
+                                              const PrimeConst& P, uint32_t (&e)[E]) {
+  constexpr int HE = E >= 8 ? E / 2 : E;
+#pragma unroll
+  for (int h = 0; h < E / HE; ++h) {
+    const size_t off = ((size_t)i << dp.log_n) + pos0 + CS * (HE / 4) * h;
+    uint32_t b1[HE], b2[HE], a1[HE], a2[HE];
+    load_runs<HE, CS>(b1, a.x0 + off);
+    load_runs<HE, CS>(b2, a.x1 + off);
+    if (u == 0) {
+#pragma unroll
+      for (int k = 0; k < HE; ++k)
+        e[HE * h + k] = MONT ? redc64((uint64_t)b1[k] * b2[k], P.q, P.m) : mulmod(b1[k], b2[k], P);
+    } else {
+      load_runs<HE, CS>(a1, a.x0 + a.poly_stride0 + off);
+      load_runs<HE, CS>(a2, a.x1 + a.poly_stride1 + off);
+#pragma unroll
+      for (int k = 0; k < HE; ++k)
+        e[HE * h + k] = MONT ? redc64((uint64_t)a1[k] * b2[k] + (uint64_t)a2[k] * b1[k], P.q, P.m)
+                             : addm(mulmod(a1[k], b2[k], P), mulmod(a2[k], b1[k], P), P.q);
+    }
+  }
+}
+template <int E, int CS>
+__device__ __forceinline__ void ks_extra(const DevParams& dp, const KsArgs& a, int u, int i, uint32_t pos0,
+                                         const PrimeConst& P, uint32_t (&e)[E]) {
+  if (a.extra == 1) {
+    ks_extra_runs<E, CS, false>(dp, a, u, i, pos0, P, e);
+  } else if (a.extra == 2 && u == 0) {
+    const uint32_t* sb = a.x0 + ((size_t)i << dp.log_n);
+#pragma unroll
+    for (int k = 0; k < E; ++k) e[k] = __ldg(sb + auto_src(pos0 + CS * (k / 4) + k % 4, a.galois, dp.log_n));
+  } else {
+#pragma unroll
+    for (int k = 0; k < E; ++k) e[k] = 0;
+  }
+}
 
 // ModDown epilogue after the NTT rows of z (launch limb y = u n + i):
 // out_u[i] = (A_u[i] - z) P^-1 + extra_u[i].
@@ -402,24 +425,22 @@ struct EpiModDown {
     prefetch_l2(A + u * a_stride + ((size_t)i << dp.log_n) + pos0);
     prefetch_tensor_inputs(dp, a, u, i, pos0);
   }
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int y, int2,
-                                             uint32_t pos0) const {
+  template <int E, int CS>
+  __device__ __forceinline__ void early(const DevParams& dp, uint32_t (&op)[E], int y, uint32_t pos0) const {
+    load_runs<E, CS>(op, A + (y / a.n) * a_stride + ((size_t)(y % a.n) << dp.log_n) + pos0);
+  }
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], const uint32_t (&acc)[E], int y, int2,
+                                        uint32_t pos0) const {
     const int n = a.n, u = y / n, i = y % n;
     const PrimeConst P = dp.pc[a.base + i];
     const uint2 pinv = dp.ks.dn_pinv[a.base + i];
-    const size_t limb = (size_t)i << dp.log_n;
+    uint32_t e[E];
+    ks_extra<E, CS>(dp, a, u, i, pos0, P, e);
 #pragma unroll
-    for (int c = 0; c < E / 4; ++c) {
-      const uint32_t p = pos0 + 4 * c;
-      uint32_t acc[4], e[4], z[4];
-      load_vec<4>(acc, A + u * a_stride + limb + p);
-      ks_extra4(dp, a, u, i, p, P, e);
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        z[k] = addm(csub(shoup(acc[k] - x[4 * c + k] + P.q, pinv.x, pinv.y, P.q), P.q), e[k], P.q);
-      store_vec<4>(a.out + u * a.out_stride + limb + p, z);
-    }
+    for (int k = 0; k < E; ++k)
+      x[k] = addm(csub(shoup(acc[k] - x[k] + P.q, pinv.x, pinv.y, P.q), P.q), e[k], P.q);
+    store_runs<E, CS>(a.out + u * a.out_stride + ((size_t)i << dp.log_n) + pos0, x);
   }
 };
 
@@ -433,57 +454,30 @@ struct SrcModDownTop {
   KsArgs a;
   const uint32_t* A;
   size_t a_stride;
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int y, int2 lm,
-                                             uint32_t pos0) const {
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], int y, int2 lm, uint32_t pos0) const {
     const int two_alpha = 2 * dp.alpha;
     if (y < two_alpha) {
-      load_vec<E>(x, A + ((size_t)lm.x << dp.log_n) + pos0);
+      load_runs<E, CS>(x, A + ((size_t)lm.x << dp.log_n) + pos0);
       return;
     }
     const int u = y - two_alpha, top = a.n - 1;
     const PrimeConst P = dp.pc[top];
     const uint2 pinv = dp.ks.dn_pinv[top];
+    uint32_t e[E];
+    load_runs<E, CS>(x, A + u * a_stride + ((size_t)top << dp.log_n) + pos0);
+    ks_extra<E, CS>(dp, a, u, top, pos0, P, e);
 #pragma unroll
-    for (int c = 0; c < E / 4; ++c) {
-      const uint32_t p = pos0 + 4 * c;
-      uint32_t acc[4], e[4];
-      load_vec<4>(acc, A + u * a_stride + ((size_t)top << dp.log_n) + p);
-      ks_extra4(dp, a, u, top, p, P, e);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) x[4 * c + k] = addm(csub(shoup(acc[k], pinv.x, pinv.y, P.q), P.q), e[k], P.q);
-    }
+    for (int k = 0; k < E; ++k) x[k] = addm(csub(shoup(x[k], pinv.x, pinv.y, P.q), P.q), e[k], P.q);
   }
 };
-
-// HMult's d0 = b1 b2 (u = 0) or d1 = a1 b2 + a2 b1 (u = 1) at limb i, times
-// 2^-32: the 64-bit product (or sum of two, below 2 q^2 < 2^32 q) through one
-// unsigned Montgomery reduction, in [0, 2q]; the caller's constant carries
-// the 2^32 back.
-__device__ __forceinline__ void tensor_d4_mont(const DevParams& dp, const KsArgs& a, int u, int i, uint32_t p0,
-                                               const PrimeConst& P, uint32_t (&e)[4]) {
-  const size_t off = ((size_t)i << dp.log_n) + p0;
-  uint32_t b1[4], b2[4];
-  load_vec<4>(b1, a.x0 + off);
-  load_vec<4>(b2, a.x1 + off);
-  if (u == 0) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) e[k] = redc64((uint64_t)b1[k] * b2[k], P.q, P.m);
-  } else {
-    uint32_t a1[4], a2[4];
-    load_vec<4>(a1, a.x0 + a.poly_stride0 + off);
-    load_vec<4>(a2, a.x1 + a.poly_stride1 + off);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) e[k] = redc64((uint64_t)a1[k] * b2[k] + (uint64_t)a2[k] * b1[k], P.q, P.m);
-  }
-}
 
 // Output of the fused ModDown + rescale after the NTT rows of the conversion
 // w (launch limb y = u top + i, top = l): out_u[i] = (A_u[i] - w)(P q_l)^-1 +
 // extra_u[i] q_l^-1, d0/d1 re-formed from the four input limbs (at the
 // three-pass rows' 24 warps per SM their loads hide: 39 us against 23 + 23
 // us as rows then a streaming kernel). For HMult (extra = 1) the products are
-// reduced once (tensor_d4_mont) and q_l^-1 2^32 restores their scale.
+// reduced once (ks_extra_runs) and q_l^-1 2^32 restores their scale.
 struct EpiRsOut {
   KsArgs a;
   const uint32_t* A;
@@ -493,28 +487,26 @@ struct EpiRsOut {
     prefetch_l2(A + u * a_stride + ((size_t)i << dp.log_n) + pos0);
     prefetch_tensor_inputs(dp, a, u, i, pos0);
   }
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int y, int2,
-                                             uint32_t pos0) const {
+  template <int E, int CS>
+  __device__ __forceinline__ void early(const DevParams& dp, uint32_t (&op)[E], int y, uint32_t pos0) const {
+    const int top = a.n - 1;
+    load_runs<E, CS>(op, A + (y / top) * a_stride + ((size_t)(y % top) << dp.log_n) + pos0);
+  }
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], const uint32_t (&acc)[E], int y, int2,
+                                        uint32_t pos0) const {
     const int top = a.n - 1, u = y / top, i = y % top;
     const PrimeConst P = dp.pc[i];
     const bool mont = a.extra == 1;
     const uint2 pq = dp.ks.dn_pqinv[top * dp.L + i],
                 qi = mont ? dp.ks.rs_qinv_r[top * dp.L + i] : dp.ks.rs_qinv[top * dp.L + i];
-    const size_t limb = (size_t)i << dp.log_n;
+    uint32_t e[E];
+    if (mont) ks_extra_runs<E, CS, true>(dp, a, u, i, pos0, P, e);
+    else ks_extra<E, CS>(dp, a, u, i, pos0, P, e);
 #pragma unroll
-    for (int c = 0; c < E / 4; ++c) {
-      const uint32_t p = pos0 + 4 * c;
-      uint32_t acc[4], e[4], z[4];
-      load_vec<4>(acc, A + u * a_stride + limb + p);
-      if (mont) tensor_d4_mont(dp, a, u, i, p, P, e);
-      else ks_extra4(dp, a, u, i, p, P, e);
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        z[k] = addm(csub(shoup(acc[k] - x[4 * c + k] + P.q, pq.x, pq.y, P.q), P.q),
-                    csub(shoup(e[k], qi.x, qi.y, P.q), P.q), P.q);
-      store_vec<4>(a.out + u * a.out_stride + limb + p, z);
-    }
+    for (int k = 0; k < E; ++k)
+      x[k] = addm(csub(shoup(acc[k] - x[k] + P.q, pq.x, pq.y, P.q), P.q), csub(shoup(e[k], qi.x, qi.y, P.q), P.q), P.q);
+    store_runs<E, CS>(a.out + u * a.out_stride + ((size_t)i << dp.log_n) + pos0, x);
   }
 };
 
@@ -532,30 +524,28 @@ struct EpiMmOut {
     prefetch_l2(A + u * a_stride + ((size_t)old_limb << dp.log_n) + pos0);
     prefetch_tensor_inputs(dp, a, u, old_limb, pos0);
   }
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int y, int2,
-                                             uint32_t pos0) const {
+  template <int E, int CS>
+  __device__ __forceinline__ void early(const DevParams& dp, uint32_t (&op)[E], int y, uint32_t pos0) const {
+    const int old_limb = m.epi[y % m.n1].old_limb;
+    if (old_limb >= 0) load_runs<E, CS>(op, A + (y / m.n1) * a_stride + ((size_t)old_limb << dp.log_n) + pos0);
+  }
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], const uint32_t (&acc)[E], int y, int2,
+                                        uint32_t pos0) const {
     const int u = y / m.n1, t = y % m.n1;
     const MmEpi e = m.epi[t];
     const PrimeConst P = dp.pc[m.s1 + t];
     const uint32_t q = P.q;
 #pragma unroll
-    for (int c = 0; c < E / 4; ++c) {
-      const uint32_t p = pos0 + 4 * c;
-      uint32_t w[4];
+    for (int k = 0; k < E; ++k) x[k] = csub(q - csub(shoup(x[k], e.c3.x, e.c3.y, q), q), q);
+    if (e.old_limb >= 0) {
+      uint32_t ex[E];
+      ks_extra<E, CS>(dp, a, u, e.old_limb, pos0, P, ex);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) w[k] = csub(q - csub(shoup(x[4 * c + k], e.c3.x, e.c3.y, q), q), q);
-      if (e.old_limb >= 0) {
-        uint32_t acc[4], ex[4];
-        load_vec<4>(acc, A + u * a_stride + ((size_t)e.old_limb << dp.log_n) + p);
-        ks_extra4(dp, a, u, e.old_limb, p, P, ex);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          w[k] = addm(addm(w[k], csub(shoup(acc[k], e.c1.x, e.c1.y, q), q), q),
-                      csub(shoup(ex[k], e.c2.x, e.c2.y, q), q), q);
-      }
-      store_vec<4>(a.out + u * a.out_stride + ((size_t)t << dp.log_n) + p, w);
+      for (int k = 0; k < E; ++k)
+        x[k] = addm(addm(x[k], csub(shoup(acc[k], e.c1.x, e.c1.y, q), q), q), csub(shoup(ex[k], e.c2.x, e.c2.y, q), q), q);
     }
+    store_runs<E, CS>(a.out + u * a.out_stride + ((size_t)t << dp.log_n) + pos0, x);
   }
 };
 
@@ -570,22 +560,19 @@ struct EpiRescale {
   __device__ __forceinline__ void prefetch(const DevParams& dp, int y, uint32_t pos0) const {
     prefetch_l2(in + (y / top) * sin + ((size_t)(y % top) << dp.log_n) + pos0);
   }
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int y, int2,
-                                             uint32_t pos0) const {
+  template <int E, int CS>
+  __device__ __forceinline__ void early(const DevParams& dp, uint32_t (&op)[E], int y, uint32_t pos0) const {
+    load_runs<E, CS>(op, in + (y / top) * sin + ((size_t)(y % top) << dp.log_n) + pos0);
+  }
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], const uint32_t (&cv)[E], int y, int2,
+                                        uint32_t pos0) const {
     const int u = y / top, i = y % top;
-    const PrimeConst P = dp.pc[i];
+    const uint32_t q = dp.pc[i].q;
     const uint2 qinv = dp.ks.rs_qinv[top * dp.L + i];
-    const size_t limb = (size_t)i << dp.log_n;
 #pragma unroll
-    for (int c = 0; c < E / 4; ++c) {
-      const uint32_t p = pos0 + 4 * c;
-      uint32_t cv[4], z[4];
-      load_vec<4>(cv, in + u * sin + limb + p);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) z[k] = csub(shoup(cv[k] - x[4 * c + k] + P.q, qinv.x, qinv.y, P.q), P.q);
-      store_vec<4>(out + u * sout + limb + p, z);
-    }
+    for (int k = 0; k < E; ++k) x[k] = csub(shoup(cv[k] - x[k] + q, qinv.x, qinv.y, q), q);
+    store_runs<E, CS>(out + u * sout + ((size_t)i << dp.log_n) + pos0, x);
   }
 };
 
@@ -596,22 +583,17 @@ struct SrcMerged {
   KsArgs a;
   const uint32_t* A;
   int ext;
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int, int2 lm,
-                                             uint32_t pos0) const {
-    load_vec<E>(x, A + ((size_t)lm.x << dp.log_n) + pos0);
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], int, int2 lm, uint32_t pos0) const {
+    load_runs<E, CS>(x, A + ((size_t)lm.x << dp.log_n) + pos0);
     const int u = lm.x / ext, t = lm.x % ext;
     if (t >= a.n) return;
     const PrimeConst P = dp.pc[lm.y];
     const uint2 pinv = dp.ks.dn_pinv[lm.y];
+    uint32_t e[E];
+    ks_extra<E, CS>(dp, a, u, t, pos0, P, e);
 #pragma unroll
-    for (int c = 0; c < E / 4; ++c) {
-      uint32_t e[4];
-      ks_extra4(dp, a, u, t, pos0 + 4 * c, P, e);
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        x[4 * c + k] = addm(csub(shoup(x[4 * c + k], pinv.x, pinv.y, P.q), P.q), e[k], P.q);
-    }
+    for (int k = 0; k < E; ++k) x[k] = addm(csub(shoup(x[k], pinv.x, pinv.y, P.q), P.q), e[k], P.q);
   }
 };
 
@@ -621,10 +603,9 @@ struct SrcDrop {
   const uint32_t* in;
   size_t sin;
   const int2* drop;
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int y, int2,
-                                             uint32_t pos0) const {
-    load_vec<E>(x, in + (y & 1) * sin + ((size_t)drop[y >> 1].x << dp.log_n) + pos0);
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], int y, int2, uint32_t pos0) const {
+    load_runs<E, CS>(x, in + (y & 1) * sin + ((size_t)drop[y >> 1].x << dp.log_n) + pos0);
   }
 };
 
@@ -641,27 +622,26 @@ struct EpiRational {
     const int old_limb = r.epi[y % r.n1].old_limb;
     if (old_limb >= 0) prefetch_l2(in + (y / r.n1) * sin + ((size_t)old_limb << dp.log_n) + pos0);
   }
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int y, int2,
-                                             uint32_t pos0) const {
+  template <int E, int CS>
+  __device__ __forceinline__ void early(const DevParams& dp, uint32_t (&op)[E], int y, uint32_t pos0) const {
+    const int old_limb = r.epi[y % r.n1].old_limb;
+    if (old_limb >= 0) {
+      load_runs<E, CS>(op, in + (y / r.n1) * sin + ((size_t)old_limb << dp.log_n) + pos0);
+    } else {
+#pragma unroll
+      for (int k = 0; k < E; ++k) op[k] = 0;
+    }
+  }
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], const uint32_t (&cv)[E], int y, int2,
+                                        uint32_t pos0) const {
     const int u = y / r.n1, i = y % r.n1;
     const uint32_t q = dp.pc[r.s1 + i].q;
     const RrEpi e = r.epi[i];
-    const uint32_t* c = e.old_limb >= 0 ? in + u * sin + ((size_t)e.old_limb << dp.log_n) : nullptr;
-    uint32_t* o = out + u * sout + ((size_t)i << dp.log_n);
 #pragma unroll
-    for (int k4 = 0; k4 < E / 4; ++k4) {
-      const uint32_t p = pos0 + 4 * k4;
-      uint32_t cv[4] = {0, 0, 0, 0}, z[4];
-      if (c) load_vec<4>(cv, c + p);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t a = csub(shoup(cv[k], e.ta_tdi.x, e.ta_tdi.y, q), q);
-        const uint32_t b = csub(shoup(x[4 * k4 + k], e.tdi.x, e.tdi.y, q), q);
-        z[k] = csub(a + q - b, q);
-      }
-      store_vec<4>(o + p, z);
-    }
+    for (int k = 0; k < E; ++k)
+      x[k] = csub(csub(shoup(cv[k], e.ta_tdi.x, e.ta_tdi.y, q), q) + q - csub(shoup(x[k], e.tdi.x, e.tdi.y, q), q), q);
+    store_runs<E, CS>(out + u * sout + ((size_t)i << dp.log_n) + pos0, x);
   }
 };
 
@@ -744,7 +724,6 @@ template <class G>
 static void moddown_tail(const DevParams& dp, const Scratch& sc, const KsArgs& a, const uint32_t* A,
                          size_t a_stride, cudaStream_t st) {
   const int n = a.n, alpha = dp.alpha;
-  const size_t limb = (size_t)1 << dp.log_n;
   // P limbs n .. n+alpha-1 of both accumulators -> S [2][alpha] (compact)
   launch_rows_g<G>(dp, true, A, sc.S, 2 * alpha,
                    LimbMap{nullptr, n, n + alpha, n, dp.L, alpha, (int)(a_stride >> dp.log_n)}, true, st);
@@ -1022,7 +1001,7 @@ int tune_columns(const DevParams& dp, const Scratch& sc, Tuning& tu, const KsArg
     if constexpr (G::W == 1024) {
       int best_p = 3;
       float best_ms = -1.f;
-      for (int passes : {3, 2, 4, 5}) {  // form 6 (twiddles in shared memory): by hand only
+      for (int passes : {3, 2}) {
         if (rc != CKKS_OK || lvl.rows_cnt < 1) break;
         DevParams dv = dp;
         dv.rows_passes = passes;

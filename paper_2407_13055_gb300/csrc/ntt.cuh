@@ -177,6 +177,22 @@ __device__ __forceinline__ void load_vec(uint32_t (&x)[E], const uint32_t* __res
   }
 }
 
+// Loads/stores of E / 4 runs of four consecutive words, run c at p + CS c.
+template <int E, int CS>
+__device__ __forceinline__ void load_runs(uint32_t (&x)[E], const uint32_t* __restrict__ p) {
+#pragma unroll
+  for (int c = 0; c < E / 4; ++c) {
+    const uint4 t = __ldg(reinterpret_cast<const uint4*>(p + CS * c));
+    x[4 * c] = t.x; x[4 * c + 1] = t.y; x[4 * c + 2] = t.z; x[4 * c + 3] = t.w;
+  }
+}
+template <int E, int CS>
+__device__ __forceinline__ void store_runs(uint32_t* p, const uint32_t (&x)[E]) {
+#pragma unroll
+  for (int c = 0; c < E / 4; ++c)
+    *reinterpret_cast<uint4*>(p + CS * c) = make_uint4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+}
+
 // Streaming load (read once: cache-streaming, evict-first policy).
 template <int E>
 __device__ __forceinline__ void load_vec_stream(uint32_t (&x)[E], const uint32_t* __restrict__ p) {

@@ -10,7 +10,6 @@
 #include "geo.cuh"
 #include "internal.h"
 #include "pdl.cuh"
-#include "tc.cuh"
 
 namespace ckks {
 
@@ -157,28 +156,34 @@ __device__ __forceinline__ void load_pass_b_twiddles(uint2 (&tw)[E - 1], const u
 }
 
 // Where a forward row phase puts its results, and where an inverse row phase
-// gets its inputs. A thread holds the E consecutive device positions
-// pos0 .. pos0 + E - 1 of its row (B layout: pos0 = h W + E jj) of launch
-// limb y, whose data limb and prime are lm = map(y). The plain forms store to
+// gets its inputs. A thread holds E device positions of its row of launch
+// limb y, whose data limb and prime are lm = map(y): E / 4 runs of four
+// consecutive words, run c at pos0 + CS c. CS = 4 is the B layout (E
+// consecutive words from pos0 = h W + E jj); CS = 128 is the warp's 512 words
+// dealt out in 16-byte units, lane after lane, so that each access of a warp
+// covers 512 consecutive bytes. The plain forms store to
 // / load from a limb array; the key-switch kernels supply fused ones (input
 // preparation before the iNTT, ModDown and rescale epilogues after the NTT).
+// An epilogue's early() loads its first operand; the three-pass kernel calls it
+// before the last pass, so that the load's latency passes behind it.
 struct RowStore {
   uint32_t* dst;
   int compact;  // write launch limb y at dst + y N instead of at data limb lm.x
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int y, int2 lm,
-                                             uint32_t pos0) const {
+  template <int E, int CS>
+  __device__ __forceinline__ void early(const DevParams&, uint32_t (&)[E], int, uint32_t) const {}
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], const uint32_t (&)[E], int y, int2 lm,
+                                        uint32_t pos0) const {
     const size_t dl = compact ? (size_t)y : (size_t)lm.x;
-    store_vec<E>(dst + (dl << dp.log_n) + pos0, x);
+    store_runs<E, CS>(dst + (dl << dp.log_n) + pos0, x);
   }
 };
 
 struct RowLoad {
   const uint32_t* src;
-  template <int E>
-  __device__ __forceinline__ void operator()(const DevParams& dp, uint32_t (&x)[E], int, int2 lm,
-                                             uint32_t pos0) const {
-    load_vec<E>(x, src + ((size_t)lm.x << dp.log_n) + pos0);
+  template <int E, int CS>
+  __device__ __forceinline__ void apply(const DevParams& dp, uint32_t (&x)[E], int, int2 lm, uint32_t pos0) const {
+    load_runs<E, CS>(x, src + ((size_t)lm.x << dp.log_n) + pos0);
   }
 };
 
@@ -219,7 +224,9 @@ __global__ void __launch_bounds__(G::RT) k_rows_fwd_t(DevParams dp, const uint32
 #pragma unroll
     for (int i = 0; i < G::ER; ++i) x[i] = normalize<false>(x[i], q);
   }
-  epi(dp, x, (int)blockIdx.y, lm, (uint32_t)(h * G::W + G::ER * jj));
+  uint32_t op[G::ER];
+  epi.template early<G::ER, 4>(dp, op, (int)blockIdx.y, (uint32_t)(h * G::W + G::ER * jj));
+  epi.template apply<G::ER, 4>(dp, x, op, (int)blockIdx.y, lm, (uint32_t)(h * G::W + G::ER * jj));
 }
 
 // Inverse row phase: the source gives B-layout values in [0, q) (NTT domain);
@@ -242,7 +249,7 @@ __global__ void __launch_bounds__(G::RT) k_rows_inv_t(DevParams dp, Src src, uin
   pdl_wait();
   pdl_trigger();
   uint32_t x[G::ER];
-  src(dp, x, (int)blockIdx.y, lm, (uint32_t)(h * G::W + G::ER * jj));
+  src.template apply<G::ER, 4>(dp, x, (int)blockIdx.y, lm, (uint32_t)(h * G::W + G::ER * jj));
   uint32_t* b = buf + r * G::ROWBUF;
   if (q < (1u << 30)) {
     gs_pass_reg<G::ER, true>(x, twb, q);
@@ -268,30 +275,92 @@ __global__ void __launch_bounds__(G::RT) k_rows_inv_t(DevParams dp, Src src, uin
 //   A layout (pass A):  thread t, value i < 16:         e = t + 64 i
 //   B layout (pass B):  thread t, group g < 2, i < 8:   e = 64 (t >> 2) + 8 i + 2 (t & 3) + g
 //   C layout (pass C):  thread t, group g < 2, i < 8:   e = 16 t + 8 g + i
-// so the row's forward output (C layout) is the same B-layout run of 16
-// consecutive words per thread that the epilogues expect. Forward stage k
-// (0 .. 9 of the row) uses twiddle (H + h) 2^k + (e >> (10 - k)); pass A's
-// 15 depend on the row only and are staged in shared memory, pass B's on
-// o = t >> 2 (base (H + h) 16 + o), pass C's on the group (base (H + h) 128
-// + 2 t + g). Launch bounds of 6 blocks of 4 warps per SM (80 registers):
-// 24 resident warps, against 16 for the two-pass form at 128 registers.
-// Transposes go through one 1024-word buffer per row with an XOR
-// swizzle of the bank bits by bits 5-8 of e, conflict-free for the three
-// access patterns (32 consecutive e; fixed i, g over a warp in B; fixed i
-// over a warp in C).
+//   dealt-out layout:   thread t, run c < 4, k < 4:     e = 512 (t >> 5) + 128 c + 4 (t & 31) + k
+// Forward stage k (0 .. 9 of the row) uses twiddle (H + h) 2^k + (e >> (10 - k));
+// pass A's 15 depend on the row only and are staged in shared memory, pass B's
+// on o = t >> 2 (base (H + h) 16 + o), pass C's on the group (base (H + h) 128
+// + 2 t + g; read from a copy of the table in the order the threads take them).
+//
+// Transposes go through one padded buffer per row, element e at word e + 8
+// (e >> 6) + 4 ((e >> 5) & 1): 32-bit accesses in A, 64-bit in B, 128-bit in C
+// and dealt out are all conflict-free, and a thread's accesses of a layout
+// differ by constants (no address arithmetic; an XOR swizzle with 32-bit
+// accesses took one operation per element and 64 accesses instead of 44).
+// Global memory is read and written in A or dealt out, whole 128- and 512-byte
+// runs per access of a warp: with the C layout's 16 consecutive words per
+// thread each 16-byte access touched 32 sectors and used half of each.
+//
+// Launch bounds of 12 blocks of 2 warps per SM (80 registers): 24 resident
+// warps, against 16 for the two-pass form at 128 registers (14 blocks: 17.6 us
+// for the ModUp rows of two-row blocks, 10: 18.6).
+//
+// Bound and figures (ModUp rows at the top level, 40 primes, dnum = 3, 122
+// limbs, launched back to back): 24.4 us with the XOR swizzle, table-order
+// twiddles and strided stores (21.2 with the shorter butterflies and whole-run
+// stores) -> 16.5; 32 MB in, 32 MB out and 62 MB of twiddles, all in L2. A warp
+// issues in half the cycles; loads from L2 are the largest stall, the multiply
+// pipe is half busy. Whole operations: HRot 133.3 -> 122.0 us, HMult + rescale
+// 153.1 -> 140.1.
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ int row3_swz(int e) {
-  const int b5 = (e >> 5) & 1, b6 = (e >> 6) & 1, b7 = (e >> 7) & 1, b8 = (e >> 8) & 1;
-  return e ^ ((b8 << 4) | (b7 << 3) | (b5 << 2) | (b8 << 1) | b6);
+constexpr int kRow3Words = 1152;
+__device__ __forceinline__ int row3_a(int t) { return t + 4 * (t >> 5); }                  // + 72 i
+__device__ __forceinline__ int row3_b(int t) { return 72 * (t >> 2) + 2 * (t & 3); }      // + 8 i + 4 (i >> 2) + g
+__device__ __forceinline__ int row3_c(int t) { return 72 * (t >> 2) + 16 * (t & 3) + 4 * ((t >> 1) & 1); }  // + 8 g + i
+__device__ __forceinline__ int row3_dealt(int t) { return 512 * (t >> 5) + 4 * (t & 31); }  // element of run 0
+__device__ __forceinline__ int row3_d(int t) {                                            // + 144 c
+  const int e = row3_dealt(t);
+  return e + 8 * (e >> 6) + 4 * ((e >> 5) & 1);
 }
-__device__ __forceinline__ int row3_eb(int t, int g, int i) { return 64 * (t >> 2) + 8 * i + 2 * (t & 3) + g; }
 
-// Pass-B and pass-C twiddles of thread t in row h: local stage s, block b at
-// entry (2^s - 1) + b, global index base 2^s + b.
+__device__ __forceinline__ void row3_put_a(uint32_t* b, int t, const uint32_t (&x)[16]) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) b[row3_a(t) + 72 * i] = x[i];
+}
+__device__ __forceinline__ void row3_get_a(const uint32_t* b, int t, uint32_t (&x)[16]) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) x[i] = b[row3_a(t) + 72 * i];
+}
+__device__ __forceinline__ void row3_put_b(uint32_t* b, int t, const uint32_t (&y0)[8], const uint32_t (&y1)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    *reinterpret_cast<uint2*>(b + row3_b(t) + 8 * i + 4 * (i >> 2)) = make_uint2(y0[i], y1[i]);
+}
+__device__ __forceinline__ void row3_get_b(const uint32_t* b, int t, uint32_t (&y0)[8], uint32_t (&y1)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint2 v = *reinterpret_cast<const uint2*>(b + row3_b(t) + 8 * i + 4 * (i >> 2));
+    y0[i] = v.x;
+    y1[i] = v.y;
+  }
+}
+// Four 16-byte units from word `at`, STEP words apart.
+template <int STEP>
+__device__ __forceinline__ void row3_put4(uint32_t* at, const uint32_t (&x)[16]) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    *reinterpret_cast<uint4*>(at + STEP * c) = make_uint4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+}
+template <int STEP>
+__device__ __forceinline__ void row3_get4(const uint32_t* at, uint32_t (&x)[16]) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const uint4 v = *reinterpret_cast<const uint4*>(at + STEP * c);
+    x[4 * c] = v.x; x[4 * c + 1] = v.y; x[4 * c + 2] = v.z; x[4 * c + 3] = v.w;
+  }
+}
+__device__ __forceinline__ void row3_split(const uint32_t (&x)[16], uint32_t (&y0)[8], uint32_t (&y1)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    y0[i] = x[i];
+    y1[i] = x[8 + i];
+  }
+}
+
+// Pass-B twiddles of thread t in row h: local stage s, block b at entry
+// (2^s - 1) + b, global index base 2^s + b.
 template <int H>
-__device__ __forceinline__ void row3_load_twiddles(uint2 (&tb)[7], uint2 (&tc)[2][7], const uint2* __restrict__ t,
-                                                   int h, int tid) {
+__device__ __forceinline__ void row3_twiddles_b(uint2 (&tb)[7], const uint2* __restrict__ t, int h, int tid) {
   const uint32_t bb = (uint32_t)(H + h) * 16 + (tid >> 2);
   tb[0] = __ldg(t + bb);
   {
@@ -305,24 +374,29 @@ __device__ __forceinline__ void row3_load_twiddles(uint2 (&tb)[7], uint2 (&tc)[2
     tb[3 + 2 * k] = make_uint2(v.x, v.y);
     tb[4 + 2 * k] = make_uint2(v.z, v.w);
   }
-  // pass C: the two groups' blocks are adjacent, so each stage is one run
-  const uint32_t bc = (uint32_t)(H + h) * 128 + 2 * tid;
-  {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(t + bc));
-    tc[0][0] = make_uint2(v.x, v.y);
-    tc[1][0] = make_uint2(v.z, v.w);
-  }
+}
+
+// Pass-C twiddles of thread t in row h, from the table in thread order
+// (DevParams::twc / itwc): unit k of thread t at (h 7 + k) 64 + t, unit 0 =
+// stage 0 of groups 0 and 1, 1 + g = stage 1 of group g, 3 + 2g and 4 + 2g =
+// stage 2 of group g. Whole 512-byte runs per access; in table order the
+// accesses of stages 1 and 2 were 32 and 64 bytes apart (84 instead of 28
+// 128-byte lines per warp).
+__device__ __forceinline__ void row3_twiddles_c(uint2 (&tc)[2][7], const uint4* __restrict__ t, int h, int tid) {
+  uint4 v[7];
 #pragma unroll
-  for (int k = 0; k < 2; ++k) {  // stage 1: entries 2 bc + 2 g + b
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(t + 2 * bc) + k);
-    tc[k][1] = make_uint2(v.x, v.y);
-    tc[k][2] = make_uint2(v.z, v.w);
-  }
+  for (int k = 0; k < 7; ++k) v[k] = __ldg(t + (h * 7 + k) * 64 + tid);
+  tc[0][0] = make_uint2(v[0].x, v[0].y);
+  tc[1][0] = make_uint2(v[0].z, v[0].w);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {  // stage 2: entries 4 bc + 4 g + b
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(t + 4 * bc) + k);
-    tc[k >> 1][3 + 2 * (k & 1)] = make_uint2(v.x, v.y);
-    tc[k >> 1][4 + 2 * (k & 1)] = make_uint2(v.z, v.w);
+  for (int g = 0; g < 2; ++g) {
+    tc[g][1] = make_uint2(v[1 + g].x, v[1 + g].y);
+    tc[g][2] = make_uint2(v[1 + g].z, v[1 + g].w);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      tc[g][3 + 2 * k] = make_uint2(v[3 + 2 * g + k].x, v[3 + 2 * g + k].y);
+      tc[g][4 + 2 * k] = make_uint2(v[3 + 2 * g + k].z, v[3 + 2 * g + k].w);
+    }
   }
 }
 
@@ -336,22 +410,27 @@ __device__ __forceinline__ void row3_stage_a(uint2* sm, const uint2* __restrict_
   }
 }
 
+constexpr int kRow3Rows = 1;  // rows per block (two: ModUp rows 17.4 us, one: 16.5; the barriers join fewer warps)
+
 template <class G, class Epi>
-__global__ void __launch_bounds__(128, 6) k_rows3_fwd_t(DevParams dp, const uint32_t* src, Epi epi, LimbMap map) {
+__global__ void __launch_bounds__(64 * kRow3Rows, 12 / kRow3Rows)
+    k_rows3_fwd_t(DevParams dp, const uint32_t* src, Epi epi, LimbMap map) {
   static_assert(G::W == 1024, "three-pass rows are for W = 1024");
-  __shared__ uint32_t buf[2][1024];
-  __shared__ uint2 twa[2][15];
+  __shared__ __align__(16) uint32_t buf[kRow3Rows][kRow3Words];
+  __shared__ uint2 twa[kRow3Rows][15];
   const int r = threadIdx.x >> 6, t = threadIdx.x & 63;
-  const int h = blockIdx.x * 2 + r;
+  const int h = blockIdx.x * kRow3Rows + r;
   const int2 lm = map(blockIdx.y);
   const uint32_t q = dp.pc[lm.y].q;
   const uint2* tw = dp.tw + ((size_t)lm.y << dp.log_n);
   uint2 tb[7], tc[2][7];
-  row3_load_twiddles<G::H>(tb, tc, tw, h, t);
+  row3_twiddles_b<G::H>(tb, tw, h, t);
+  row3_twiddles_c(tc, dp.twc + (size_t)lm.y * (G::H * 448), h, t);
   row3_stage_a<G::H>(twa[r], tw, h, t);
   __syncthreads();
   pdl_wait();
   pdl_trigger();
+  const uint32_t pos = (uint32_t)(h * 1024 + row3_dealt(t));
   if constexpr (HasPrefetch<Epi>::value) epi.prefetch(dp, (int)blockIdx.y, (uint32_t)(h * 1024 + 16 * t));
   const uint32_t* s = src + ((size_t)lm.x << dp.log_n) + (size_t)h * 1024;
   uint32_t x[16];
@@ -359,36 +438,26 @@ __global__ void __launch_bounds__(128, 6) k_rows3_fwd_t(DevParams dp, const uint
   for (int i = 0; i < 16; ++i) x[i] = s[t + 64 * i];
   uint32_t* b = buf[r];
   uint32_t y0[8], y1[8];
-  if (q < (1u << 30)) ct_pass_sm<16, true>(x, twa[r], q);
+  const bool lazy = q < (1u << 30);
+  if (lazy) ct_pass_sm<16, true>(x, twa[r], q);
   else ct_pass_sm<16, false>(x, twa[r], q);
-#pragma unroll
-  for (int i = 0; i < 16; ++i) b[row3_swz(t + 64 * i)] = x[i];
+  row3_put_a(b, t, x);
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    y0[i] = b[row3_swz(row3_eb(t, 0, i))];
-    y1[i] = b[row3_swz(row3_eb(t, 1, i))];
-  }
-  __syncthreads();
-  if (q < (1u << 30)) {
+  row3_get_b(b, t, y0, y1);
+  if (lazy) {
     ct_pass_reg<8, true>(y0, tb, q);
     ct_pass_reg<8, true>(y1, tb, q);
   } else {
     ct_pass_reg<8, false>(y0, tb, q);
     ct_pass_reg<8, false>(y1, tb, q);
   }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    b[row3_swz(row3_eb(t, 0, i))] = y0[i];
-    b[row3_swz(row3_eb(t, 1, i))] = y1[i];
-  }
+  row3_put_b(b, t, y0, y1);  // where the thread read them
+  uint32_t op[16];
+  epi.template early<16, 128>(dp, op, (int)blockIdx.y, pos);
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    y0[i] = b[row3_swz(16 * t + i)];
-    y1[i] = b[row3_swz(16 * t + 8 + i)];
-  }
-  if (q < (1u << 30)) {
+  row3_get4<4>(b + row3_c(t), x);
+  row3_split(x, y0, y1);
+  if (lazy) {
     ct_pass_reg<8, true>(y0, tc[0], q);
     ct_pass_reg<8, true>(y1, tc[1], q);
 #pragma unroll
@@ -405,36 +474,40 @@ __global__ void __launch_bounds__(128, 6) k_rows3_fwd_t(DevParams dp, const uint
       x[8 + i] = normalize<false>(y1[i], q);
     }
   }
-  epi(dp, x, (int)blockIdx.y, lm, (uint32_t)(h * 1024 + 16 * t));
+  // deal out: C layout and dealt-out runs stay in the warp's half of the row
+  row3_put4<4>(b + row3_c(t), x);
+  __syncwarp();
+  row3_get4<144>(b + row3_d(t), x);
+  epi.template apply<16, 128>(dp, x, op, (int)blockIdx.y, lm, pos);
 }
 
 template <class G, class Src>
-__global__ void __launch_bounds__(128, 6) k_rows3_inv_t(DevParams dp, Src src, uint32_t* dst, LimbMap map,
-                                                     int dst_compact) {
+__global__ void __launch_bounds__(64 * kRow3Rows, 12 / kRow3Rows)
+    k_rows3_inv_t(DevParams dp, Src src, uint32_t* dst, LimbMap map, int dst_compact) {
   static_assert(G::W == 1024, "three-pass rows are for W = 1024");
-  __shared__ uint32_t buf[2][1024];
-  __shared__ uint2 twa[2][15];
+  __shared__ __align__(16) uint32_t buf[kRow3Rows][kRow3Words];
+  __shared__ uint2 twa[kRow3Rows][15];
   const int r = threadIdx.x >> 6, t = threadIdx.x & 63;
-  const int h = blockIdx.x * 2 + r;
+  const int h = blockIdx.x * kRow3Rows + r;
   const int2 lm = map(blockIdx.y);
   const uint32_t q = dp.pc[lm.y].q;
   const uint2* itw = dp.itw + ((size_t)lm.y << dp.log_n);
   uint2 tb[7], tc[2][7];
-  row3_load_twiddles<G::H>(tb, tc, itw, h, t);
+  row3_twiddles_c(tc, dp.itwc + (size_t)lm.y * (G::H * 448), h, t);
   row3_stage_a<G::H>(twa[r], itw, h, t);
-  __syncthreads();
   pdl_wait();
   pdl_trigger();
   uint32_t x[16];
-  src(dp, x, (int)blockIdx.y, lm, (uint32_t)(h * 1024 + 16 * t));
+  src.template apply<16, 128>(dp, x, (int)blockIdx.y, lm, (uint32_t)(h * 1024 + row3_dealt(t)));
   uint32_t* b = buf[r];
+  row3_put4<144>(b + row3_d(t), x);
+  row3_twiddles_b<G::H>(tb, itw, h, t);  // not before the sources' loads: registers
+  __syncwarp();
+  row3_get4<4>(b + row3_c(t), x);
   uint32_t y0[8], y1[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    y0[i] = x[i];
-    y1[i] = x[8 + i];
-  }
-  if (q < (1u << 30)) {
+  row3_split(x, y0, y1);
+  const bool lazy = q < (1u << 30);
+  if (lazy) {
     gs_pass_reg<8, true>(y0, tc[0], q);
     gs_pass_reg<8, true>(y1, tc[1], q);
   } else {
@@ -443,32 +516,23 @@ __global__ void __launch_bounds__(128, 6) k_rows3_inv_t(DevParams dp, Src src, u
   }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    b[row3_swz(16 * t + i)] = y0[i];
-    b[row3_swz(16 * t + 8 + i)] = y1[i];
+    x[i] = y0[i];
+    x[8 + i] = y1[i];
   }
+  row3_put4<4>(b + row3_c(t), x);  // where the thread read them
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    y0[i] = b[row3_swz(row3_eb(t, 0, i))];
-    y1[i] = b[row3_swz(row3_eb(t, 1, i))];
-  }
-  __syncthreads();
-  if (q < (1u << 30)) {
+  row3_get_b(b, t, y0, y1);
+  if (lazy) {
     gs_pass_reg<8, true>(y0, tb, q);
     gs_pass_reg<8, true>(y1, tb, q);
   } else {
     gs_pass_reg<8, false>(y0, tb, q);
     gs_pass_reg<8, false>(y1, tb, q);
   }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    b[row3_swz(row3_eb(t, 0, i))] = y0[i];
-    b[row3_swz(row3_eb(t, 1, i))] = y1[i];
-  }
+  row3_put_b(b, t, y0, y1);
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 16; ++i) x[i] = b[row3_swz(t + 64 * i)];
-  if (q < (1u << 30)) gs_pass_sm<16, true>(x, twa[r], q);
+  row3_get_a(b, t, x);
+  if (lazy) gs_pass_sm<16, true>(x, twa[r], q);
   else gs_pass_sm<16, false>(x, twa[r], q);
   const size_t dl = dst_compact ? (size_t)blockIdx.y : (size_t)lm.x;
   uint32_t* o = dst + (dl << dp.log_n) + (size_t)h * 1024;
@@ -476,461 +540,37 @@ __global__ void __launch_bounds__(128, 6) k_rows3_inv_t(DevParams dp, Src src, u
   for (int i = 0; i < 16; ++i) o[t + 64 * i] = x[i];
 }
 
-// ---------------------------------------------------------------------------
-// Three-pass rows with the twiddles in shared memory. The same passes, layouts
-// and twiddle indices as k_rows3_fwd_t / k_rows3_inv_t, but the pass-B and
-// pass-C twiddles (21 pairs per thread, 42 registers there) are copied into
-// shared memory with asynchronous copies (cp.async: no registers, the copies
-// land while the thread loads its row and runs its first pass) and read from
-// there at each stage. A thread then keeps little more than its 16 values, so
-// the kernel fits 8 blocks of 4 warps per SM (64 registers, 25 KB of shared
-// memory per block): 32 resident warps against 24.
-// Layouts per row: pass A as before (15 pairs, entry (2^s - 1) + b); pass B per
-// group o = t >> 2, entry (1 << s) + b (entry 0 unused), 10 entries per group
-// so that the 8 groups of a warp fall in distinct banks; pass C per thread as
-// 7 16-byte pairs in pair-major order (pair p of thread t at [p][t]): pair 0 =
-// stage 0 of groups 0 and 1, pairs 1 + g = stage 1 of group g, pairs 3 + 2g and
-// 4 + 2g = stage 2 of group g (blocks 0-1 and 2-3), each read as one 16-byte
-// word by the thread, conflict-free across the warp.
-// ---------------------------------------------------------------------------
-
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-struct Row3Tw {
-  uint2 a[2][15];        // pass A, per row
-  uint2 b[2][16][10];    // pass B, per row and group o
-  uint4 c[2][7][64];     // pass C, per row, pair, thread
-};
-
-// Copies of thread t of row r (row h of the limb's table t): pass A by the
-// first 15 threads, pass B by the four threads of each group (one stage part
-// each), pass C by every thread (its own 7 pairs). Two commit groups: pass A,
-// then passes B and C (order `a_first`), or pass C then passes B and A.
-template <int H>
-__device__ __forceinline__ void row3s_copy_twiddles(Row3Tw& sw, const uint2* __restrict__ tw, int r, int h, int t,
-                                                    bool a_first) {
-  auto copy_a = [&]() {
-    if (t < 15) {
-      const int s = 31 - __clz(t + 1);
-      const int b = t + 1 - (1 << s);
-      cp_async8(&sw.a[r][t], tw + ((uint32_t)(H + h) << s) + b);
-    }
-  };
-  auto copy_b = [&]() {
-    const int o = t >> 2, part = t & 3;
-    const uint32_t bb = (uint32_t)(H + h) * 16 + o;
-    if (part == 0) cp_async8(&sw.b[r][o][1], tw + bb);
-    else if (part == 1) cp_async16(&sw.b[r][o][2], tw + 2 * bb);
-    else cp_async16(&sw.b[r][o][4 + 2 * (part - 2)], tw + 4 * bb + 2 * (part - 2));
-  };
-  auto copy_c = [&]() {
-    const uint32_t bc = (uint32_t)(H + h) * 128 + 2 * t;
-    cp_async16(&sw.c[r][0][t], tw + bc);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) cp_async16(&sw.c[r][1 + k][t], tw + 2 * bc + 2 * k);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) cp_async16(&sw.c[r][3 + k][t], tw + 4 * bc + 2 * k);
-  };
-  if (a_first) {
-    copy_a();
-    cp_async_commit();
-    copy_b();
-    copy_c();
-  } else {
-    copy_c();
-    cp_async_commit();
-    copy_b();
-    copy_a();
-  }
-  cp_async_commit();
-}
-
-// Pass B on both groups, twiddle of stage s, block b at w[(1 << s) + b].
-template <bool LAZY>
-__device__ __forceinline__ void row3s_ct_b(uint32_t (&y0)[8], uint32_t (&y1)[8], const uint2* w, uint32_t q) {
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    const int half = 8 >> (s + 1);
-#pragma unroll
-    for (int b = 0; b < (1 << s); ++b) {
-      const uint2 tw = w[(1 << s) + b];
-#pragma unroll
-      for (int k = 0; k < half; ++k) {
-        const int i0 = b * 2 * half + k;
-        ct_bfly<LAZY>(y0[i0], y0[i0 + half], tw.x, tw.y, q);
-        ct_bfly<LAZY>(y1[i0], y1[i0 + half], tw.x, tw.y, q);
-      }
-    }
-  }
-}
-
-template <bool LAZY>
-__device__ __forceinline__ void row3s_gs_b(uint32_t (&y0)[8], uint32_t (&y1)[8], const uint2* w, uint32_t q) {
-#pragma unroll
-  for (int s = 2; s >= 0; --s) {
-    const int half = 8 >> (s + 1);
-#pragma unroll
-    for (int b = 0; b < (1 << s); ++b) {
-      const uint2 tw = w[(1 << s) + b];
-#pragma unroll
-      for (int k = 0; k < half; ++k) {
-        const int i0 = b * 2 * half + k;
-        gs_bfly<LAZY>(y0[i0], y0[i0 + half], tw.x, tw.y, q);
-        gs_bfly<LAZY>(y1[i0], y1[i0 + half], tw.x, tw.y, q);
-      }
-    }
-  }
-}
-
-// Twiddle pair of group g, stage s, block b from the thread's pass-C pairs
-// (c[p * 64] = pair p).
-__device__ __forceinline__ uint2 row3s_c_tw(const uint4* c, int g, int s, int b) {
-  const uint4 v = s == 0 ? c[0] : s == 1 ? c[(1 + g) * 64] : c[(3 + 2 * g + (b >> 1)) * 64];
-  const bool hi = s == 0 ? g == 1 : (b & 1) == 1;
-  return hi ? make_uint2(v.z, v.w) : make_uint2(v.x, v.y);
-}
-
-template <bool LAZY>
-__device__ __forceinline__ void row3s_ct_c(uint32_t (&y0)[8], uint32_t (&y1)[8], const uint4* c, uint32_t q) {
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    const int half = 8 >> (s + 1);
-#pragma unroll
-    for (int b = 0; b < (1 << s); ++b) {
-      const uint2 w0 = row3s_c_tw(c, 0, s, b), w1 = row3s_c_tw(c, 1, s, b);
-#pragma unroll
-      for (int k = 0; k < half; ++k) {
-        const int i0 = b * 2 * half + k;
-        ct_bfly<LAZY>(y0[i0], y0[i0 + half], w0.x, w0.y, q);
-        ct_bfly<LAZY>(y1[i0], y1[i0 + half], w1.x, w1.y, q);
-      }
-    }
-  }
-}
-
-template <bool LAZY>
-__device__ __forceinline__ void row3s_gs_c(uint32_t (&y0)[8], uint32_t (&y1)[8], const uint4* c, uint32_t q) {
-#pragma unroll
-  for (int s = 2; s >= 0; --s) {
-    const int half = 8 >> (s + 1);
-#pragma unroll
-    for (int b = 0; b < (1 << s); ++b) {
-      const uint2 w0 = row3s_c_tw(c, 0, s, b), w1 = row3s_c_tw(c, 1, s, b);
-#pragma unroll
-      for (int k = 0; k < half; ++k) {
-        const int i0 = b * 2 * half + k;
-        gs_bfly<LAZY>(y0[i0], y0[i0 + half], w0.x, w0.y, q);
-        gs_bfly<LAZY>(y1[i0], y1[i0 + half], w1.x, w1.y, q);
-      }
-    }
-  }
-}
-
-template <class G, class Epi>
-__global__ void __launch_bounds__(128, 8) k_rows3s_fwd_t(DevParams dp, const uint32_t* src, Epi epi, LimbMap map) {
-  static_assert(G::W == 1024, "three-pass rows are for W = 1024");
-  __shared__ uint32_t buf[2][1024];
-  __shared__ __align__(16) Row3Tw sw;
-  const int r = threadIdx.x >> 6, t = threadIdx.x & 63;
-  const int h = blockIdx.x * 2 + r;
-  const int2 lm = map(blockIdx.y);
-  const uint32_t q = dp.pc[lm.y].q;
-  row3s_copy_twiddles<G::H>(sw, dp.tw + ((size_t)lm.y << dp.log_n), r, h, t, true);
-  pdl_wait();
-  pdl_trigger();
-  const uint32_t* s = src + ((size_t)lm.x << dp.log_n) + (size_t)h * 1024;
-  uint32_t x[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) x[i] = s[t + 64 * i];
-  cp_async_wait<1>();
-  __syncthreads();
-  uint32_t* b = buf[r];
-  uint32_t y0[8], y1[8];
-  const bool lazy = q < (1u << 30);
-  if (lazy) ct_pass_sm<16, true>(x, sw.a[r], q);
-  else ct_pass_sm<16, false>(x, sw.a[r], q);
-#pragma unroll
-  for (int i = 0; i < 16; ++i) b[row3_swz(t + 64 * i)] = x[i];
-  cp_async_wait<0>();
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    y0[i] = b[row3_swz(row3_eb(t, 0, i))];
-    y1[i] = b[row3_swz(row3_eb(t, 1, i))];
-  }
-  __syncthreads();
-  const uint2* wb = sw.b[r][t >> 2];
-  if (lazy) row3s_ct_b<true>(y0, y1, wb, q);
-  else row3s_ct_b<false>(y0, y1, wb, q);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    b[row3_swz(row3_eb(t, 0, i))] = y0[i];
-    b[row3_swz(row3_eb(t, 1, i))] = y1[i];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    y0[i] = b[row3_swz(16 * t + i)];
-    y1[i] = b[row3_swz(16 * t + 8 + i)];
-  }
-  const uint4* wc = &sw.c[r][0][t];
-  if (lazy) {
-    row3s_ct_c<true>(y0, y1, wc, q);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      x[i] = normalize<true>(y0[i], q);
-      x[8 + i] = normalize<true>(y1[i], q);
-    }
-  } else {
-    row3s_ct_c<false>(y0, y1, wc, q);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      x[i] = normalize<false>(y0[i], q);
-      x[8 + i] = normalize<false>(y1[i], q);
-    }
-  }
-  epi(dp, x, (int)blockIdx.y, lm, (uint32_t)(h * 1024 + 16 * t));
-}
-
-template <class G, class Src>
-__global__ void __launch_bounds__(128, 8) k_rows3s_inv_t(DevParams dp, Src src, uint32_t* dst, LimbMap map,
-                                                      int dst_compact) {
-  static_assert(G::W == 1024, "three-pass rows are for W = 1024");
-  __shared__ uint32_t buf[2][1024];
-  __shared__ __align__(16) Row3Tw sw;
-  const int r = threadIdx.x >> 6, t = threadIdx.x & 63;
-  const int h = blockIdx.x * 2 + r;
-  const int2 lm = map(blockIdx.y);
-  const uint32_t q = dp.pc[lm.y].q;
-  row3s_copy_twiddles<G::H>(sw, dp.itw + ((size_t)lm.y << dp.log_n), r, h, t, false);
-  pdl_wait();
-  pdl_trigger();
-  uint32_t x[16];
-  src(dp, x, (int)blockIdx.y, lm, (uint32_t)(h * 1024 + 16 * t));
-  uint32_t* b = buf[r];
-  uint32_t y0[8], y1[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    y0[i] = x[i];
-    y1[i] = x[8 + i];
-  }
-  const bool lazy = q < (1u << 30);
-  cp_async_wait<1>();  // own pass-C pairs (read by this thread only)
-  const uint4* wc = &sw.c[r][0][t];
-  if (lazy) row3s_gs_c<true>(y0, y1, wc, q);
-  else row3s_gs_c<false>(y0, y1, wc, q);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    b[row3_swz(16 * t + i)] = y0[i];
-    b[row3_swz(16 * t + 8 + i)] = y1[i];
-  }
-  cp_async_wait<0>();
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    y0[i] = b[row3_swz(row3_eb(t, 0, i))];
-    y1[i] = b[row3_swz(row3_eb(t, 1, i))];
-  }
-  __syncthreads();
-  const uint2* wb = sw.b[r][t >> 2];
-  if (lazy) row3s_gs_b<true>(y0, y1, wb, q);
-  else row3s_gs_b<false>(y0, y1, wb, q);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    b[row3_swz(row3_eb(t, 0, i))] = y0[i];
-    b[row3_swz(row3_eb(t, 1, i))] = y1[i];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 16; ++i) x[i] = b[row3_swz(t + 64 * i)];
-  if (lazy) gs_pass_sm<16, true>(x, sw.a[r], q);
-  else gs_pass_sm<16, false>(x, sw.a[r], q);
-  const size_t dl = dst_compact ? (size_t)blockIdx.y : (size_t)lm.x;
-  uint32_t* o = dst + (dl << dp.log_n) + (size_t)h * 1024;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) o[t + 64 * i] = x[i];
-}
-
-// Three-pass forward rows with the input staged by bulk copies: a block
-// takes RP consecutive row pairs of one limb; the next pairs' 8 KB of input
-// (two contiguous rows) stream into a second shared buffer with
-// cp.async.bulk (one thread issues, an mbarrier counts the bytes) while the
-// current pair is transformed, so the loads' latency overlaps the
-// arithmetic. The staging buffer of a pair also holds its transposes. Every
-// wait is bounded by dp.wait_limit (expired: status word, the block stops
-// after draining its own copies). In-place use (src == the epilogue's
-// destination) is safe: a block reads and writes only its own rows.
-template <class G, class Epi, int RP>
-__global__ void __launch_bounds__(128, 5) k_rows3_fwd_bulk(DevParams dp, const uint32_t* src, Epi epi, LimbMap map) {
-  static_assert(G::W == 1024, "three-pass rows are for W = 1024");
-  __shared__ __align__(128) uint32_t buf[2][2][1024];
-  __shared__ uint2 twa[2][15];
-  __shared__ __align__(8) uint64_t bar[2];
-  const int r = threadIdx.x >> 6, t = threadIdx.x & 63;
-  const int2 lm = map(blockIdx.y);
-  const uint32_t q = dp.pc[lm.y].q;
-  const uint2* tw = dp.tw + ((size_t)lm.y << dp.log_n);
-  const uint32_t* s0 = src + ((size_t)lm.x << dp.log_n);
-  const int pair0 = blockIdx.x * RP;
-  if (threadIdx.x == 0) {
-    tc::mbar_init(tc::smem_u32(&bar[0]), 1);
-    tc::mbar_init(tc::smem_u32(&bar[1]), 1);
-    tc::mbar_init_fence();
-  }
-  uint2 tb[7], tc_[2][7];
-  row3_load_twiddles<G::H>(tb, tc_, tw, 2 * pair0 + r, t);
-  row3_stage_a<G::H>(twa[r], tw, 2 * pair0 + r, t);
-  __syncthreads();
-  pdl_wait();
-  pdl_trigger();
-  uint32_t issued = 0;  // thread 0: copies issued (pair k goes to buffer k & 1)
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < 2 && k < RP; ++k) {
-      const uint32_t b = tc::smem_u32(&bar[k]);
-      tc::mbar_expect_tx(b, 8192);
-      tc::bulk_g2s(tc::smem_u32(buf[k]), s0 + (size_t)(pair0 + k) * 2048, 8192, b);
-      ++issued;
-    }
-  }
-  uint32_t waited = 0;
-  for (int k = 0; k < RP; ++k) {
-    const int h = 2 * (pair0 + k) + r;
-    if (k > 0) {
-      row3_load_twiddles<G::H>(tb, tc_, tw, h, t);
-      row3_stage_a<G::H>(twa[r], tw, h, t);
-    }
-    const bool ok = tc::mbar_wait(tc::smem_u32(&bar[k & 1]), (uint32_t)((k >> 1) & 1), dp.wait_limit);
-    if (__syncthreads_or(!ok)) {
-      if (threadIdx.x == 0) tc::report_timeout(dp.status);
-      break;
-    }
-    ++waited;
-    uint32_t* b = buf[k & 1][r];
-    uint32_t x[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) x[i] = b[t + 64 * i];
-    uint32_t y0[8], y1[8];
-    if (q < (1u << 30)) ct_pass_sm<16, true>(x, twa[r], q);
-    else ct_pass_sm<16, false>(x, twa[r], q);
-    __syncthreads();  // every thread read its input before the transposes overwrite it
-#pragma unroll
-    for (int i = 0; i < 16; ++i) b[row3_swz(t + 64 * i)] = x[i];
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      y0[i] = b[row3_swz(row3_eb(t, 0, i))];
-      y1[i] = b[row3_swz(row3_eb(t, 1, i))];
-    }
-    __syncthreads();
-    if (q < (1u << 30)) {
-      ct_pass_reg<8, true>(y0, tb, q);
-      ct_pass_reg<8, true>(y1, tb, q);
-    } else {
-      ct_pass_reg<8, false>(y0, tb, q);
-      ct_pass_reg<8, false>(y1, tb, q);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      b[row3_swz(row3_eb(t, 0, i))] = y0[i];
-      b[row3_swz(row3_eb(t, 1, i))] = y1[i];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      y0[i] = b[row3_swz(16 * t + i)];
-      y1[i] = b[row3_swz(16 * t + 8 + i)];
-    }
-    // the buffer and the pass-A twiddles are free once every thread has read
-    // them: the next copy into this buffer may start
-    tc::fence_proxy_async();
-    __syncthreads();
-    if (threadIdx.x == 0 && k + 2 < RP) {
-      const uint32_t bb = tc::smem_u32(&bar[k & 1]);
-      tc::mbar_expect_tx(bb, 8192);
-      tc::bulk_g2s(tc::smem_u32(buf[k & 1]), s0 + (size_t)(pair0 + k + 2) * 2048, 8192, bb);
-      ++issued;
-    }
-    if (q < (1u << 30)) {
-      ct_pass_reg<8, true>(y0, tc_[0], q);
-      ct_pass_reg<8, true>(y1, tc_[1], q);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        x[i] = normalize<true>(y0[i], q);
-        x[8 + i] = normalize<true>(y1[i], q);
-      }
-    } else {
-      ct_pass_reg<8, false>(y0, tc_[0], q);
-      ct_pass_reg<8, false>(y1, tc_[1], q);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        x[i] = normalize<false>(y0[i], q);
-        x[8 + i] = normalize<false>(y1[i], q);
-      }
-    }
-    epi(dp, x, (int)blockIdx.y, lm, (uint32_t)(h * 1024 + 16 * t));
-  }
-  // after a timeout: let the copies still in flight land before the block's
-  // shared memory is released
-  if (threadIdx.x == 0)
-    for (uint32_t k = waited; k < issued; ++k)
-      tc::mbar_wait(tc::smem_u32(&bar[k & 1]), (k >> 1) & 1, 1ll << 32);
-}
-
+// At N = 2^16 rows_passes = 2 selects the two-pass kernels, anything else the
+// three-pass ones.
 template <class G, class Epi>
 inline void launch_rows_fwd(const DevParams& dp, const uint32_t* src, const Epi& epi, int limbs, LimbMap map,
                             cudaStream_t st) {
   if (limbs <= 0) return;
-  bool three = false;
+  count_launch(1);
   if constexpr (G::W == 1024) {
-    if (dp.rows_passes == 4 || dp.rows_passes == 5) {
-      if (dp.rows_passes == 4)
-        launch_pdl(dp.pdl, k_rows3_fwd_bulk<G, Epi, 2>, dim3(G::H / 4, limbs), dim3(128), 0, st, dp, src, epi, map);
-      else
-        launch_pdl(dp.pdl, k_rows3_fwd_bulk<G, Epi, 4>, dim3(G::H / 8, limbs), dim3(128), 0, st, dp, src, epi, map);
-      three = true;
-    } else if (dp.rows_passes == 6) {
-      launch_pdl(dp.pdl, k_rows3s_fwd_t<G, Epi>, dim3(G::H / 2, limbs), dim3(128), 0, st, dp, src, epi, map);
-      three = true;
-    } else if (dp.rows_passes != 2) {
-      launch_pdl(dp.pdl, k_rows3_fwd_t<G, Epi>, dim3(G::H / 2, limbs), dim3(128), 0, st, dp, src, epi, map);
-      three = true;
+    if (dp.rows_passes != 2) {
+      launch_pdl(dp.pdl, k_rows3_fwd_t<G, Epi>, dim3(G::H / kRow3Rows, limbs), dim3(64 * kRow3Rows), 0, st, dp, src,
+                 epi, map);
+      return;
     }
   }
-  if (!three)
-    launch_pdl(dp.pdl, k_rows_fwd_t<G, Epi>, dim3(G::H / G::RPC, limbs), dim3(G::RT), 0, st, dp, src, epi, map);
-  count_launch(1);
+  launch_pdl(dp.pdl, k_rows_fwd_t<G, Epi>, dim3(G::H / G::RPC, limbs), dim3(G::RT), 0, st, dp, src, epi, map);
 }
 
 template <class G, class Src>
 inline void launch_rows_inv(const DevParams& dp, const Src& srcf, uint32_t* dst, int limbs, LimbMap map,
                             bool dst_compact, cudaStream_t st) {
   if (limbs <= 0) return;
-  bool three = false;
+  count_launch(1);
   if constexpr (G::W == 1024) {
-    if (dp.rows_passes == 6) {
-      launch_pdl(dp.pdl, k_rows3s_inv_t<G, Src>, dim3(G::H / 2, limbs), dim3(128), 0, st, dp, srcf, dst, map,
-                 dst_compact ? 1 : 0);
-      three = true;
-    } else if (dp.rows_passes != 2) {
-      launch_pdl(dp.pdl, k_rows3_inv_t<G, Src>, dim3(G::H / 2, limbs), dim3(128), 0, st, dp, srcf, dst, map,
-                 dst_compact ? 1 : 0);
-      three = true;
+    if (dp.rows_passes != 2) {
+      launch_pdl(dp.pdl, k_rows3_inv_t<G, Src>, dim3(G::H / kRow3Rows, limbs), dim3(64 * kRow3Rows), 0, st, dp, srcf,
+                 dst, map, dst_compact ? 1 : 0);
+      return;
     }
   }
-  if (!three)
-    launch_pdl(dp.pdl, k_rows_inv_t<G, Src>, dim3(G::H / G::RPC, limbs), dim3(G::RT), 0, st, dp, srcf, dst, map,
-               dst_compact ? 1 : 0);
-  count_launch(1);
+  launch_pdl(dp.pdl, k_rows_inv_t<G, Src>, dim3(G::H / G::RPC, limbs), dim3(G::RT), 0, st, dp, srcf, dst, map,
+             dst_compact ? 1 : 0);
 }
 
 template <class G>
