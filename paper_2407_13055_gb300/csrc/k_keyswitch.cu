@@ -147,6 +147,8 @@ __device__ __forceinline__ void keymult_quad(const DevParams& dp, const KsArgs& 
   const int g0 = a.base / alpha;  // first active digit of the window
   const PrimeConst P = dp.pc[id];
   uint32_t x[D][4], e0[D][4], e1[D][4];
+  const AutoQuad src(p0, a.galois, dp.log_n);
+  uint4 raw[D];
   // (streaming the key before the wait kept every key word live across it:
   // 86 registers and a third of the occupancy, so the wait comes first)
   if (wait_dep) {
@@ -157,13 +159,16 @@ __device__ __forceinline__ void keymult_quad(const DevParams& dp, const KsArgs& 
   for (int j = 0; j < D; ++j) {
     const int lo = max(0, (g0 + j) * alpha - a.base), hi = min(n, (g0 + j + 1) * alpha - a.base);
     const uint32_t* tj = T + ((size_t)(j * ext + t) << dp.log_n);
-    if (t >= lo && t < hi) {
-      ks_input4(dp, a, t, p0, x[j]);
-    } else if (a.hoisted) {
+    const bool own = t >= lo && t < hi;
+    if (a.hoisted) {
       // ModUp commutes with the automorphism exactly (centered BConv), so
-      // phi(ModUp(a)) is a gather from the ModUp limbs of a
-#pragma unroll
-      for (int k = 0; k < 4; ++k) x[j][k] = __ldg(tj + auto_src(p0 + k, a.galois, dp.log_n));
+      // phi(ModUp(a)) is a gather from the ModUp limbs of a. The quads are
+      // put in order after the key's loads are under way: in order here, digit
+      // by digit, took 18.3 us for two digits at level 24, word by word 16.2,
+      // this 16.0 (and the plain path at level 39 26.5 -> 24.2)
+      raw[j] = src.load(own ? a.x0 + a.poly_stride0 + ((size_t)t << dp.log_n) : tj);
+    } else if (own) {
+      ks_input4(dp, a, t, p0, x[j]);
     } else {
       load_vec<4>(x[j], tj + p0);
     }
@@ -177,6 +182,10 @@ __device__ __forceinline__ void keymult_quad(const DevParams& dp, const KsArgs& 
   for (int j = 0; j < D; ++j) {
     load_vec_stream<4>(e0[j], a.evk + ((size_t)(((g0 + j) * 2 + 0) * ext_top + key_limb) << dp.log_n) + p0);
     load_vec_stream<4>(e1[j], a.evk + ((size_t)(((g0 + j) * 2 + 1) * ext_top + key_limb) << dp.log_n) + p0);
+  }
+  if (a.hoisted) {
+#pragma unroll
+    for (int j = 0; j < D; ++j) src.order(raw[j], x[j]);
   }
   // acc_u = sum_j x_j e_j[u] 2^-32 mod q with one reduction per output: the
   // products (x < 2^31, e < q) are summed in 64 bits, three of them at most
@@ -228,9 +237,30 @@ static void launch_keymult(int digits, dim3 g, int th, cudaStream_t st, const De
 //   acc_u[t] = sum_i pt_i[t] (.) sum_j phi_i(ModUp_j(a))[t] (.) evk_i[j][u][t],
 // the automorphism read as a gather from the shared ModUp limbs of a (own
 // digit limbs: from a itself). The plaintexts are in the extended basis, so
-// the sum stays in Q_l P until one ModDown. A = [2][n + alpha][N].
+// the sum stays in Q_l P until one ModDown. At the ciphertext limbs the sum
+// of the terms that are not key-switched,
+//   B_0 = sum_i pt_i (.) phi_i(b),   B_1 = sum_{r_i = 0} pt_i (.) a,
+// is added times P: ModDown subtracts a conversion of the P limbs, where P B
+// is 0, and divides by P, so it comes out as B exactly. The plaintexts are
+// then read once (a kernel of its own after the ModDown read their Q limbs
+// again: 52 us of 445 for 16 terms at level 33). A = [2][n + alpha][N].
+//
+// Sums are kept in 64 bits below 2^32 q (fold64): per term the digits' products
+// fold, one Montgomery reduction (the key's factor cancels it), times the
+// plaintext, fold. Digits one after the other at 64 registers and four blocks
+// per SM (3 or 5 blocks: 1 % and 5 % slower), each load a full quad. Bound by
+// the keys: 16 terms at level 33 stream 1.13 GB of keys and 0.2 GB of
+// plaintexts, 199 us at the copy rate. Measured there: 261 us, and 52 us for
+// the other terms after the ModDown, -> 244 us for both; the operation 391.7 ->
+// 329 us.
+__device__ __forceinline__ uint32_t reduce_sum(uint64_t s, const PrimeConst& P) {  // s < 2^32 q -> [0, q)
+  const uint32_t t = csub(csub(redc64(s, P.q, P.m), P.q), P.q);                    // s 2^-32
+  return fix_signed(smr((int64_t)t * P.r2c, P.q, P.m), P.q);
+}
+
 template <int D>
-__global__ void k_lt_keymult(DevParams dp, KsArgs a, LtArgs lt, const uint32_t* T, uint32_t* A) {
+__global__ void __launch_bounds__(256, 4) k_lt_keymult(DevParams dp, KsArgs a, const __grid_constant__ LtArgs lt,
+                                                    const uint32_t* T, uint32_t* A) {
   pdl_wait();
   pdl_trigger();
   const int t = blockIdx.y;
@@ -240,39 +270,79 @@ __global__ void k_lt_keymult(DevParams dp, KsArgs a, LtArgs lt, const uint32_t* 
   const int g0 = a.base / alpha;
   const PrimeConst P = dp.pc[id];
   const uint32_t p0 = stream_pos();
-  const uint32_t* ain = a.x0 + a.poly_stride0 + ((size_t)t << dp.log_n);
-  uint32_t acc0[4] = {0, 0, 0, 0}, acc1[4] = {0, 0, 0, 0};
+  const size_t tl = (size_t)t << dp.log_n;
+  const bool q_limb = t < n;
+  const uint32_t* a_limb = a.x0 + a.poly_stride0 + tl;
+  uint64_t s0[4] = {0, 0, 0, 0}, s1[4] = {0, 0, 0, 0}, sb[4] = {0, 0, 0, 0};
+  uint32_t plain[4] = {0, 0, 0, 0};  // P B_1
+  const int64_t pr = q_limb ? dp.ks.rs_mat[id * (alpha + 1) + alpha] : 0;  // [P 2^32] centered
+  if (q_limb && lt.rotated < lt.count) {
+    for (int i = 0; i < lt.count; ++i) {
+      if (lt.evk[i]) continue;
+      uint32_t w[4], v[4], b[4];
+      load_vec<4>(w, lt.pt[i] + tl + p0);
+      load_vec<4>(v, a_limb + p0);
+      load_vec<4>(b, a.x0 + tl + p0);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        s1[k] = fold64(s1[k] + (uint64_t)v[k] * w[k], P.mont);
+        sb[k] = fold64(sb[k] + (uint64_t)b[k] * w[k], P.mont);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      plain[k] = fix_signed(smr(reduce_sum(s1[k], P) * pr, P.q, P.m), P.q);
+      s1[k] = 0;
+    }
+  }
   for (int i = 0; i < lt.count; ++i) {
     const uint32_t* evk = lt.evk[i];
     if (!evk) continue;
-    const uint32_t g = lt.galois[i];
-    uint32_t x[D][4], e0[D][4], e1[D][4], w[4];
+    const AutoQuad src(p0, lt.galois[i], dp.log_n);
+    uint64_t d0[4] = {0, 0, 0, 0}, d1[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int j = 0; j < D; ++j) {
+      uint32_t x[4], e0[4], e1[4];
+      load_vec_stream<4>(e0, evk + ((size_t)(((g0 + j) * 2 + 0) * ext_top + key_limb) << dp.log_n) + p0);
+      load_vec_stream<4>(e1, evk + ((size_t)(((g0 + j) * 2 + 1) * ext_top + key_limb) << dp.log_n) + p0);
       const int lo = max(0, (g0 + j) * alpha - a.base), hi = min(n, (g0 + j + 1) * alpha - a.base);
-      const uint32_t* src = (t >= lo && t < hi) ? ain : T + ((size_t)(j * ext + t) << dp.log_n);
+      src.order(src.load(t >= lo && t < hi ? a_limb : T + ((size_t)(j * ext + t) << dp.log_n)), x);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) x[j][k] = __ldg(src + auto_src(p0 + k, g, dp.log_n));
-      load_vec_stream<4>(e0[j], evk + ((size_t)(((g0 + j) * 2 + 0) * ext_top + key_limb) << dp.log_n) + p0);
-      load_vec_stream<4>(e1[j], evk + ((size_t)(((g0 + j) * 2 + 1) * ext_top + key_limb) << dp.log_n) + p0);
-    }
-    const int pl = t < n ? t : lt.pt_p[i] + (t - n);
-    load_vec<4>(w, lt.pt[i] + ((size_t)pl << dp.log_n) + p0);
-    uint32_t s0[4] = {0, 0, 0, 0}, s1[4] = {0, 0, 0, 0};
-#pragma unroll
-    for (int j = 0; j < D; ++j)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        s0[k] = addm(s0[k], fix_signed(mont_mul(x[j][k], e0[j][k], P.q, P.m), P.q), P.q);
-        s1[k] = addm(s1[k], fix_signed(mont_mul(x[j][k], e1[j][k], P.q, P.m), P.q), P.q);
+      for (int k = 0; k < 4; ++k) {  // three products fit before the first fold (keymult_quad)
+        d0[k] += (uint64_t)x[k] * e0[k];
+        d1[k] += (uint64_t)x[k] * e1[k];
+        if (j >= 2 || j == D - 1) {
+          d0[k] = fold64(d0[k], P.mont);
+          d1[k] = fold64(d1[k], P.mont);
+        }
       }
+    }
+    uint32_t w[4];
+    load_vec<4>(w, lt.pt[i] + ((size_t)(q_limb ? t : lt.pt_p[i] + (t - n)) << dp.log_n) + p0);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      acc0[k] = addm(acc0[k], mulmod(s0[k], w[k], P), P.q);
-      acc1[k] = addm(acc1[k], mulmod(s1[k], w[k], P), P.q);
+      // redc64 is in [0, 2q]: its product stays below 2^32 q beside the folded sum
+      s0[k] = fold64(s0[k] + (uint64_t)redc64(d0[k], P.q, P.m) * w[k], P.mont);
+      s1[k] = fold64(s1[k] + (uint64_t)redc64(d1[k], P.q, P.m) * w[k], P.mont);
+    }
+    if (q_limb) {
+      uint32_t b[4];
+      src.order(src.load(a.x0 + tl), b);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) sb[k] = fold64(sb[k] + (uint64_t)b[k] * w[k], P.mont);
     }
   }
-  store_vec<4>(A + ((size_t)t << dp.log_n) + p0, acc0);
+  uint32_t acc0[4], acc1[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    acc0[k] = reduce_sum(s0[k], P);
+    acc1[k] = reduce_sum(s1[k], P);
+    if (q_limb) {
+      acc0[k] = addm(acc0[k], fix_signed(smr(reduce_sum(sb[k], P) * pr, P.q, P.m), P.q), P.q);
+      acc1[k] = addm(acc1[k], plain[k], P.q);
+    }
+  }
+  store_vec<4>(A + tl + p0, acc0);
   store_vec<4>(A + ((size_t)(ext + t) << dp.log_n) + p0, acc1);
 }
 
@@ -288,12 +358,9 @@ static void launch_lt_keymult(int digits, dim3 g, int th, cudaStream_t st, const
   }
 }
 
-// Linear transform epilogue, limb i of output poly u:
-//   out_0 = (A_0 - Z_0) P^-1 + sum_i pt_i (.) phi_i(b)      (accumulated automorphisms, Par. 4)
-//   out_1 = (A_1 - Z_1) P^-1 + sum_{i: r_i = 0} pt_i (.) a
-// ks = 0 (no rotated term): the key-switch part is zero and A, Z are not read.
-__global__ void k_lt_epilogue(DevParams dp, KsArgs a, LtArgs lt, const uint32_t* Z, const uint32_t* A,
-                              size_t a_stride, int ks) {
+// Linear transform without a rotated term, limb i of output poly u:
+//   out_0 = sum_i pt_i (.) b,   out_1 = sum_i pt_i (.) a.
+__global__ void k_lt_plain(DevParams dp, KsArgs a, const __grid_constant__ LtArgs lt) {
   pdl_wait();
   pdl_trigger();
   const int n = a.n;
@@ -301,27 +368,12 @@ __global__ void k_lt_epilogue(DevParams dp, KsArgs a, LtArgs lt, const uint32_t*
   const PrimeConst P = dp.pc[a.base + i];
   const uint32_t p0 = stream_pos();
   const size_t off = ((size_t)i << dp.log_n) + p0;
+  const uint32_t* src = a.x0 + u * a.poly_stride0;
   uint32_t z[4] = {0, 0, 0, 0};
-  if (ks) {
-    const uint2 pinv = dp.ks.dn_pinv[a.base + i];
-    uint32_t acc[4];
-    load_vec<4>(z, Z + ((size_t)(u * n + i) << dp.log_n) + p0);
-    load_vec<4>(acc, A + u * a_stride + off);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) z[k] = csub(shoup(acc[k] - z[k] + P.q, pinv.x, pinv.y, P.q), P.q);
-  }
-  const uint32_t* src = a.x0 + u * a.poly_stride0 + ((size_t)i << dp.log_n);
   for (int t = 0; t < lt.count; ++t) {
-    const bool plain = lt.evk[t] == nullptr;
-    if (u == 1 && !plain) continue;
     uint32_t w[4], v[4];
     load_vec<4>(w, lt.pt[t] + off);
-    if (plain) {
-      load_vec<4>(v, src + p0);
-    } else {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = __ldg(src + auto_src(p0 + k, lt.galois[t], dp.log_n));
-    }
+    load_vec<4>(v, src + off);
 #pragma unroll
     for (int k = 0; k < 4; ++k) z[k] = addm(z[k], mulmod(w[k], v[k], P), P.q);
   }
@@ -1072,9 +1124,8 @@ void launch_hoisted_rotations(const DevParams& dp0, const Scratch& sc, const KsA
 }
 
 // Linear transform (Par. 5): ModUp of a once, KeyMult + MAC of all rotated
-// terms with their extended plaintexts in one kernel, one ModDown of the
-// sum, and the epilogue adding the plaintext-weighted automorphisms of b
-// (and pt (.) a for unrotated terms).
+// terms with their extended plaintexts (and the other terms times P) in one
+// kernel, one ModDown of the sum.
 void launch_linear_transform(const DevParams& dp0, const Scratch& sc, const KsArgs& a, const LtArgs& lt,
                              cudaStream_t st) {
   const DevParams dp = tuned_rows(dp0, sc, a.tix);
@@ -1100,20 +1151,13 @@ void launch_linear_transform(const DevParams& dp0, const Scratch& sc, const KsAr
       launch_lt_keymult(digits, g, th, st, dp, a, lt, sc.T, sc.A);
       count_launch(1);
       prof_mark(sc, st, P_KEYMULT);
-      const size_t a_stride = (size_t)ext * limb;
-      launch_rows_g<G>(dp, true, sc.A, down.S, 2 * alpha,
-                       LimbMap{nullptr, n, n + alpha, n, dp.L, alpha, (int)(a_stride >> dp.log_n)}, true, st);
-      prof_mark(sc, st, P_MODDOWN_IN_ROWS);
-      launch_moddown_cols<G>(dp, n, a.base, a.tix, down, pick_shape<G>(sc, CK_MODDOWN, a.tix, alpha, 2 * alpha * n), st);
-      prof_mark(sc, st, P_MODDOWN_COLS);
-      launch_rows_g<G>(dp, false, down.T, down.T, 2 * n, window_map(a, dp.L), false, st);
-      prof_mark(sc, st, P_MODDOWN_ROWS);
+      moddown_tail<G>(dp, down, a, sc.A, (size_t)ext * limb, st);
+    } else {
+      stream_grid(dp.log_n, 2 * n, g, th);
+      launch_pdl(dp.pdl, k_lt_plain, g, dim3(th), 0, st, dp, a, lt);
+      count_launch(1);
+      prof_mark(sc, st, P_KS_EPILOGUE);
     }
-    stream_grid(dp.log_n, 2 * n, g, th);
-    launch_pdl(dp.pdl, k_lt_epilogue, g, dim3(th), 0, st, dp, a, lt, (const uint32_t*)down.T, (const uint32_t*)sc.A,
-               (size_t)ext * limb, lt.rotated > 0 ? 1 : 0);
-    count_launch(1);
-    prof_mark(sc, st, P_KS_EPILOGUE);
   });
 }
 
