@@ -243,6 +243,7 @@ int ckks_ctx_clone(ckks_ctx* parent, void* cuda_stream, ckks_ctx** out) {
   c->d_tables = parent->d_tables;
   c->table_bytes = 0;
   c->owns_tables = false;
+  c->enc = parent->enc;
   c->gadget_p = parent->gadget_p;
   c->device = parent->device;
   c->windowed = parent->windowed;
@@ -274,6 +275,8 @@ void ckks_ctx_destroy(ckks_ctx* ctx) {
   if (ctx->d_tables && ctx->owns_tables) cudaFree(ctx->d_tables);
   if (ctx->d_scratch) cudaFree(ctx->d_scratch);
   if (ctx->d_unfused) cudaFree(ctx->d_unfused);
+  if (ctx->d_enc) cudaFree(ctx->d_enc);
+  if (ctx->d_dec) cudaFree(ctx->d_dec);
   if (ctx->owns_tables) free_status(ctx);
   for (cudaEvent_t e : ctx->prof.ev) cudaEventDestroy(e);
   delete ctx;
@@ -856,23 +859,36 @@ int ckks_evk_import(ckks_ctx* ctx, const uint32_t* host, uint32_t galois, ckks_e
 // encoding and encryption
 // ---------------------------------------------------------------------------
 
+// Workspace of encoding and decoding: N complex values, then N / 2 slots.
+static int enc_workspace(ckks_ctx* ctx) {
+  if (ctx->d_enc) return CKKS_OK;
+  const cudaError_t e = cudaMalloc(&ctx->d_enc, (size_t)ctx->N * 3 / 2 * sizeof(double2));
+  if (e != cudaSuccess) ctx->d_enc = nullptr;
+  return e == cudaSuccess ? CKKS_OK : CKKS_ENOMEM;
+}
+
+// The slots' rounded polynomial modulo the limbs' primes, NTT domain.
+static int encode_limbs(ckks_ctx* ctx, const double* re_im, double scale, uint32_t* out, int limbs, IdMap ids) {
+  std::lock_guard<std::mutex> lock(ctx->enc_lock);
+  if (enc_workspace(ctx)) return fail(ctx, CKKS_ENOMEM, "encode scratch");
+  double2* slots = ctx->d_enc + ctx->N;
+  int rc = cuda_check(ctx, cudaMemcpyAsync(slots, re_im, (size_t)ctx->N * 8, cudaMemcpyHostToDevice, ctx->stream), "upload");
+  if (!rc) {
+    launch_encode(ctx->dp, ctx->enc, slots, ctx->d_enc, scale, ctx->stream);
+    launch_small_to_res(ctx->dp, reinterpret_cast<const int64_t*>(slots), out, limbs, ids, ctx->stream);
+    launch_ntt(ctx->dp, out, limbs, ids, false, ctx->stream);
+    rc = launched(ctx, "encode");
+  }
+  return rc ? rc : sync_check(ctx, "encode");
+}
+
 int ckks_encode(ckks_ctx* ctx, const double* re_im, int level, double scale, ckks_pt** out) {
   if (!ctx || !re_im || !out) return CKKS_EINVAL;
   if (level < 0 || level >= ctx->n_levels()) return fail(ctx, CKKS_ELEVEL, "level %d out of range", level);
-  std::vector<int64_t> m;
-  host_encode(re_im, ctx->dp.log_n, scale, m);
   int rc = pt_alloc(ctx, level, scale, out);
   if (rc) return rc;
-  DevBuf tmp;
   const int n = ctx->lvl_n(level), base = ctx->lvl_base(level);
-  rc = tmp.alloc(m.size() * 8) ? fail(ctx, CKKS_ENOMEM, "encode scratch") : CKKS_OK;
-  if (!rc) rc = cuda_check(ctx, cudaMemcpyAsync(tmp.p, m.data(), m.size() * 8, cudaMemcpyHostToDevice, ctx->stream), "upload");
-  if (!rc) {
-    launch_small_to_res(ctx->dp, tmp.as<int64_t>(), (*out)->d, n, id_ct(n, ctx->dp.L, base), ctx->stream);
-    launch_ntt(ctx->dp, (*out)->d, n, id_ct(n, ctx->dp.L, base), false, ctx->stream);
-    rc = launched(ctx, "encode");
-  }
-  if (!rc) rc = sync_check(ctx, "encode");
+  rc = encode_limbs(ctx, re_im, scale, (*out)->d, n, id_ct(n, ctx->dp.L, base));
   if (rc) {
     ckks_free(*out);
     *out = nullptr;
@@ -883,21 +899,10 @@ int ckks_encode(ckks_ctx* ctx, const double* re_im, int level, double scale, ckk
 int ckks_encode_ext(ckks_ctx* ctx, const double* re_im, int level, double scale, ckks_pt** out) {
   if (!ctx || !re_im || !out) return CKKS_EINVAL;
   if (level < 0 || level >= ctx->n_levels()) return fail(ctx, CKKS_ELEVEL, "level %d out of range", level);
-  std::vector<int64_t> m;
-  host_encode(re_im, ctx->dp.log_n, scale, m);
   const int alpha = ctx->dp.alpha, n = ctx->lvl_n(level), base = ctx->lvl_base(level);
   int rc = pt_alloc(ctx, level, scale, out, alpha);
   if (rc) return rc;
-  DevBuf tmp;
-  rc = tmp.alloc(m.size() * 8) ? fail(ctx, CKKS_ENOMEM, "encode scratch") : CKKS_OK;
-  if (!rc) rc = cuda_check(ctx, cudaMemcpyAsync(tmp.p, m.data(), m.size() * 8, cudaMemcpyHostToDevice, ctx->stream), "upload");
-  if (!rc) {
-    const IdMap ids = id_ext(n, ctx->dp.L, alpha, base);
-    launch_small_to_res(ctx->dp, tmp.as<int64_t>(), (*out)->d, n + alpha, ids, ctx->stream);
-    launch_ntt(ctx->dp, (*out)->d, n + alpha, ids, false, ctx->stream);
-    rc = launched(ctx, "encode");
-  }
-  if (!rc) rc = sync_check(ctx, "encode");
+  rc = encode_limbs(ctx, re_im, scale, (*out)->d, n + alpha, id_ext(n, ctx->dp.L, alpha, base));
   if (rc) {
     ckks_free(*out);
     *out = nullptr;
@@ -908,20 +913,28 @@ int ckks_encode_ext(ckks_ctx* ctx, const double* re_im, int level, double scale,
 int ckks_decode(ckks_ctx* ctx, const ckks_pt* pt, double* re_im_out) {
   if (!ctx || !pt || !re_im_out) return CKKS_EINVAL;
   const int n = ctx->lvl_n(pt->level), base = ctx->lvl_base(pt->level);
-  const size_t lw = limb_words(ctx);
-  DevBuf tmp;
-  if (tmp.alloc((size_t)n * lw * 4)) return fail(ctx, CKKS_ENOMEM, "decode scratch");
-  int rc = cuda_check(ctx, cudaMemcpyAsync(tmp.p, pt->d, (size_t)n * lw * 4, cudaMemcpyDeviceToDevice, ctx->stream), "copy");
+  const size_t bytes = (size_t)n * limb_words(ctx) * 4;
+  std::lock_guard<std::mutex> lock(ctx->enc_lock);
+  if (ctx->dec_limbs < n) {
+    if (ctx->d_dec) cudaFree(ctx->d_dec);
+    ctx->dec_limbs = 0;
+    if (cudaMalloc(&ctx->d_dec, bytes) != cudaSuccess) {
+      ctx->d_dec = nullptr;
+      return fail(ctx, CKKS_ENOMEM, "decode scratch");
+    }
+    ctx->dec_limbs = n;
+  }
+  if (enc_workspace(ctx)) return fail(ctx, CKKS_ENOMEM, "decode scratch");
+  double2* slots = ctx->d_enc + ctx->N;
+  int rc = cuda_check(ctx, cudaMemcpyAsync(ctx->d_dec, pt->d, bytes, cudaMemcpyDeviceToDevice, ctx->stream), "copy");
   if (rc) return rc;
-  launch_ntt(ctx->dp, tmp.as<uint32_t>(), n, id_ct(n, ctx->dp.L, base), true, ctx->stream);
+  launch_ntt(ctx->dp, ctx->d_dec, n, id_ct(n, ctx->dp.L, base), true, ctx->stream);
+  launch_decode(ctx->dp, ctx->enc, ctx->d_dec, n, base, ctx->enc.half + (size_t)pt->level * ctx->dp.L, pt->scale,
+                ctx->d_enc, slots, ctx->stream);
   rc = launched(ctx, "decode");
   if (rc) return rc;
-  std::vector<uint32_t> res((size_t)n * lw);
-  rc = cuda_check(ctx, cudaMemcpyAsync(res.data(), tmp.p, res.size() * 4, cudaMemcpyDeviceToHost, ctx->stream), "download");
-  if (!rc) rc = sync_check(ctx, "decode");
-  if (rc) return rc;
-  host_decode(res.data(), n, ctx->q.data() + base, ctx->dp.log_n, pt->scale, re_im_out);
-  return CKKS_OK;
+  rc = cuda_check(ctx, cudaMemcpyAsync(re_im_out, slots, (size_t)ctx->N * 8, cudaMemcpyDeviceToHost, ctx->stream), "download");
+  return rc ? rc : sync_check(ctx, "decode");
 }
 
 int ckks_encrypt(ckks_ctx* ctx, const ckks_sk* sk, const ckks_pt* pt, uint64_t seed, ckks_ct** out) {

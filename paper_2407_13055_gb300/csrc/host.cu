@@ -1,6 +1,5 @@
 // Host-side number theory, table construction, sampling and encoding.
 #include <cmath>
-#include <complex>
 #include <cstring>
 
 #include <algorithm>
@@ -341,103 +340,6 @@ void Sampler::ternary(int64_t* s, int n, int hw) {
     int j = i + (int)(next() % (uint64_t)(n - i));
     std::swap(idx[i], idx[j]);
     s[idx[i]] = (next() >> 63) ? 1 : -1;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Encoding: slot j <-> zeta^(5^j mod 2N), zeta = exp(i pi / N)
-// ---------------------------------------------------------------------------
-namespace {
-typedef std::complex<double> cd;
-
-// In-place radix-2 FFT: A[k] = sum_j a[j] exp(sign 2 pi i jk / n).
-void fft(std::vector<cd>& a, int sign) {
-  const int n = (int)a.size();
-  for (int i = 1, j = 0; i < n; ++i) {
-    int bit = n >> 1;
-    for (; j & bit; bit >>= 1) j ^= bit;
-    j ^= bit;
-    if (i < j) std::swap(a[i], a[j]);
-  }
-  for (int len = 2; len <= n; len <<= 1) {
-    const double ang = sign * 2 * M_PI / len;
-    for (int i = 0; i < n; i += len)
-      for (int k = 0; k < len / 2; ++k) {
-        const cd w(std::cos(ang * k), std::sin(ang * k));
-        const cd u = a[i + k], v = a[i + k + len / 2] * w;
-        a[i + k] = u + v;
-        a[i + k + len / 2] = u - v;
-      }
-  }
-}
-}  // namespace
-
-void host_encode(const double* re_im, int log_n, double scale, std::vector<int64_t>& coeffs) {
-  const int n = 1 << log_n;
-  std::vector<cd> zo(n, 0.0);  // z at zeta^(2j+1), j < N
-  uint64_t e = 1;
-  for (int j = 0; j < n / 2; ++j) {
-    const cd u(re_im[2 * j], re_im[2 * j + 1]);
-    zo[(e - 1) / 2] = u;
-    zo[(2 * n - e - 1) / 2] = std::conj(u);
-    e = e * 5 % (2 * n);
-  }
-  fft(zo, -1);  // sum_j z_(2j+1) exp(-2 pi i jk / N)
-  coeffs.resize(n);
-  for (int k = 0; k < n; ++k) {
-    const cd tw(std::cos(-M_PI * k / n), std::sin(-M_PI * k / n));
-    const double v = (zo[k] * tw).real() / n * scale;
-    coeffs[k] = (int64_t)(v < 0 ? -std::floor(-v + 0.5) : std::floor(v + 0.5));
-  }
-}
-
-void host_decode(const uint32_t* res, int nl, const uint32_t* q, int log_n, double scale, double* re_im) {
-  const int n = 1 << log_n;
-  // Garner mixed-radix digits; inv[i][j] = q_j^-1 mod q_i.
-  std::vector<uint32_t> inv((size_t)nl * nl);
-  for (int i = 0; i < nl; ++i)
-    for (int j = 0; j < i; ++j) inv[(size_t)i * nl + j] = invm(q[j] % q[i], q[i]);
-  // mixed-radix digits of (Q-1)/2, whose residues are (q_i - 1)/2
-  std::vector<uint32_t> half(nl), v(nl);
-  for (int i = 0; i < nl; ++i) {
-    uint32_t t = (q[i] - 1) / 2;
-    for (int j = 0; j < i; ++j) t = mulm((t + q[i] - half[j] % q[i]) % q[i], inv[(size_t)i * nl + j], q[i]);
-    half[i] = t;
-  }
-  std::vector<cd> m(n);
-  for (int k = 0; k < n; ++k) {
-    for (int i = 0; i < nl; ++i) {
-      uint32_t t = res[(size_t)i * n + k];
-      for (int j = 0; j < i; ++j) t = mulm((t + q[i] - v[j] % q[i]) % q[i], inv[(size_t)i * nl + j], q[i]);
-      v[i] = t;
-    }
-    bool neg = false;
-    for (int i = nl - 1; i >= 0; --i) {
-      if (v[i] != half[i]) {
-        neg = v[i] > half[i];
-        break;
-      }
-    }
-    // value = d_0 + q_0 (d_1 + q_1 (d_2 + ...)), evaluated from the top digit
-    // (Horner): the leading digits of a small value are 0 (or q_i - 1 for a
-    // negative one), so nothing overflows however many limbs there are.
-    double x = 0;
-    if (!neg) {
-      for (int i = nl - 1; i >= 0; --i) x = x * (double)q[i] + (double)v[i];
-    } else {
-      for (int i = nl - 1; i >= 0; --i) x = x * (double)q[i] + (double)(q[i] - 1 - v[i]);
-      x = -(x + 1);
-    }
-    const cd tw(std::cos(M_PI * k / n), std::sin(M_PI * k / n));
-    m[k] = x * tw;
-  }
-  fft(m, +1);  // sum_k m_k zeta^k exp(2 pi i jk / N) = value at zeta^(2j+1)
-  uint64_t e = 1;
-  for (int j = 0; j < n / 2; ++j) {
-    const cd z = m[(e - 1) / 2] / scale;
-    re_im[2 * j] = z.real();
-    re_im[2 * j + 1] = z.imag();
-    e = e * 5 % (2 * n);
   }
 }
 
@@ -831,6 +733,27 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
     }
   }
 
+  // encoding: powers of zeta = exp(i pi / N); decoding: inverses between the
+  // primes and each level's digits of (Q - 1) / 2 in mixed radix, whose
+  // residues are (q_i - 1) / 2
+  std::vector<double2> enc_tw(n);
+  for (int k = 0; k < n; ++k) enc_tw[k] = make_double2(std::cos(M_PI * k / n), std::sin(M_PI * k / n));
+  std::vector<uint2> dec_inv((size_t)L * L, make_uint2(0, 0));
+  for (int i = 0; i < L; ++i)
+    for (int j = 0; j < L; ++j)
+      if (i != j) dec_inv[(size_t)i * L + j] = shoup_pair(invm(pr[j] % pr[i], pr[i]), pr[i]);
+  std::vector<uint32_t> dec_half((size_t)nlev * L, 0);
+  for (int l = 0; l < nlev; ++l) {
+    const int s0 = ctx->lvl_first[l];
+    uint32_t* half = dec_half.data() + (size_t)l * L;
+    for (int i = 0; i < ctx->lvl_count[l]; ++i) {
+      const uint32_t q = pr[s0 + i];
+      uint32_t t = (q - 1) / 2;
+      for (int j = 0; j < i; ++j) t = mulm((t + q - half[j] % q) % q, dec_inv[(size_t)(s0 + i) * L + s0 + j].x, q);
+      half[i] = t;
+    }
+  }
+
   // one device allocation for all tables
   struct Part {
     const void* src;
@@ -866,6 +789,9 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
       {tc_tgt.data(), tc_tgt.size() * sizeof(TcTgtRec), 0},
       {twc.data(), twc.size() * sizeof(uint2), 0},
       {itwc.data(), itwc.size() * sizeof(uint2), 0},
+      {enc_tw.data(), enc_tw.size() * sizeof(double2), 0},
+      {dec_inv.data(), dec_inv.size() * sizeof(uint2), 0},
+      {dec_half.data(), dec_half.size() * sizeof(uint32_t), 0},
   };
   size_t total = 0;
   for (auto& p : parts) {
@@ -892,6 +818,9 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
   dp.itw = reinterpret_cast<const uint2*>(base + parts[2].off);
   dp.twc = reinterpret_cast<const uint4*>(base + parts[26].off);
   dp.itwc = reinterpret_cast<const uint4*>(base + parts[27].off);
+  ctx->enc = EncTables{reinterpret_cast<const double2*>(base + parts[28].off),
+                       reinterpret_cast<const uint2*>(base + parts[29].off),
+                       reinterpret_cast<const uint32_t*>(base + parts[30].off)};
   dp.ks.up_cin = reinterpret_cast<const uint2*>(base + parts[3].off);
   dp.ks.up_mat = reinterpret_cast<const int32_t*>(base + parts[4].off);
   dp.ks.up_off = reinterpret_cast<const int2*>(base + parts[5].off);

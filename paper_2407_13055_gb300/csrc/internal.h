@@ -6,6 +6,7 @@
 #include <atomic>
 #include <cstdint>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -343,6 +344,17 @@ void launch_tensor(const DevParams& dp, const uint32_t* c1, const uint32_t* c2, 
                    cudaStream_t st);
 void launch_automorph(const DevParams& dp, const uint32_t* in, uint32_t* out, int limbs, uint32_t galois,
                       cudaStream_t st);
+// k_encode.cu. Encoding: slots (N / 2 complex values) -> N rounded coefficients
+// (int64, in the slots' place). Decoding: canonical residues [nl][N] of the
+// window from prime base on (coefficient domain) -> slots. z: N values of scratch.
+struct EncTables {
+  const double2* tw;     // [N] zeta^k = exp(i pi k / N)
+  const uint2* inv;      // [L][L] (i, j < i): q_j^-1 mod q_i and its Shoup companion
+  const uint32_t* half;  // [levels][L] mixed-radix digits of (Q - 1) / 2 of the level's primes
+};
+void launch_encode(const DevParams& dp, const EncTables& et, double2* slots, double2* z, double scale, cudaStream_t st);
+void launch_decode(const DevParams& dp, const EncTables& et, const uint32_t* res, int nl, int base,
+                   const uint32_t* half, double scale, double2* z, double2* slots, cudaStream_t st);
 void launch_small_to_res(const DevParams& dp, const int64_t* v, uint32_t* out, int limbs, IdMap ids,
                          cudaStream_t st);
 // out = sign_as * a * s + c + d (mod q), limb-wise; any pointer may be null (term skipped).
@@ -455,6 +467,15 @@ struct ckks_ctx {
   void* d_scratch;
   size_t scratch_bytes;
   uint32_t* d_unfused = nullptr;  // scratch of the unfused form (allocated on its first use)
+  // Encoding and decoding: tables (the parent's, for a clone), and a workspace
+  // allocated on the first use (N complex values, N / 2 slots, the residues of
+  // the largest level decoded so far). The calls return when their kernels are
+  // done; the lock keeps calls of several threads apart.
+  ckks::EncTables enc{};
+  std::mutex enc_lock;
+  double2* d_enc = nullptr;
+  uint32_t* d_dec = nullptr;
+  int dec_limbs = 0;
   // host-side key-switching constants needed for keygen (gadget P mod prime)
   std::vector<uint2> gadget_p;  // [L + alpha] Shoup pair of [P]_{prime}
   std::string err;
@@ -546,10 +567,6 @@ bool host_is_prime(uint64_t n);
 uint32_t host_find_psi(uint32_t q, int log_n);
 int host_gen_primes(int log_n, int n_q, int n_p, uint32_t* q, uint32_t* p);
 int host_gen_prime_system_2530(int log_n, int n_p, uint32_t* q, uint32_t* p, int* first, int* count);
-// Encoding (fp64): N/2 complex slots -> N rounded integer coefficients.
-void host_encode(const double* re_im, int log_n, double scale, std::vector<int64_t>& coeffs);
-// Decoding from canonical residues [n][N] (coefficient domain).
-void host_decode(const uint32_t* res, int n, const uint32_t* q, int log_n, double scale, double* re_im);
 // Sampler (SplitMix64 stream).
 struct Sampler {
   uint64_t state;
