@@ -44,6 +44,8 @@ struct ckks_batch {
 
 namespace {
 
+constexpr size_t kL2Bytes = 100u << 20;  // of 129 MB: the keys stream through the rest
+
 int issue_one(ckks_ctx* lane, const ckks_op& o) {
   switch (o.op) {
     case CKKS_OP_HMULT:
@@ -70,8 +72,36 @@ int cuda_fail(ckks_ctx* ctx, cudaError_t e, const char* what) {
   return CKKS_ECUDA;
 }
 
-// Issue the whole list: lane l takes operations i = l mod lanes; lanes 1..
-// fork from and join back into lane 0's stream.
+// The lane of each operation: in list order, the least loaded of the lanes it
+// may use. An operation may use as many lanes as operations of its level fit
+// in the L2 side by side (the limbs of a key switch: inputs and output, ModUp,
+// accumulators), two at least: above that they push each other's limbs out
+// between their kernels, below it more lanes hide more of the launches.
+// 24 operations of one level at N = 2^16, dnum = 3 (us; 1, 2, 4, 6 lanes): level
+// 5 756, 557, 514, 511; level 10 883, 688, 686, 679; level 15 1106, 899, 997,
+// 1016; level 25 1389, 1199, 1362, 1347; level 39 2223, 2070, 2188, 2059. Four
+// lanes given, lanes in turn -> by this rule: 48 operations of levels 1 .. 39
+// 2866 -> 2602, 33 of levels 10 .. 16 1247 -> 1180, 27 of levels 5 .. 8 660 ->
+// 658 (with 129 MB for the L2 2700, 1194, 662).
+std::vector<int> assign_lanes(const ckks_batch* b) {
+  const ckks::DevParams& dp = b->ctx->dp;
+  const size_t nl = b->lanes.size();
+  std::vector<int> lane(b->ops.size());
+  std::vector<size_t> load(nl, 0);  // in 0.6 us at N = 2^16
+  for (size_t i = 0; i < b->ops.size(); ++i) {
+    const ckks_op& o = b->ops[i];
+    const size_t n = b->ctx->lvl_n(o.a->level), digits = (n + dp.alpha - 1) / dp.alpha;
+    const size_t bytes = (6 * n + (digits + 2) * (n + dp.alpha)) * 4 << dp.log_n;
+    const size_t use = std::min(nl, std::max<size_t>(2, kL2Bytes / bytes));
+    const size_t at = std::min_element(load.begin(), load.begin() + use) - load.begin();
+    const bool key_switch = o.op == CKKS_OP_HMULT || o.op == CKKS_OP_HROT || o.op == CKKS_OP_HCONJ;
+    lane[i] = (int)at;
+    load[at] += key_switch ? 60 + 4 * n : o.op == CKKS_OP_RESCALE ? 20 + n : 8 + n / 2;
+  }
+  return lane;
+}
+
+// Issue the whole list; lanes 1.. fork from and join back into lane 0's stream.
 int issue_all(ckks_batch* b) {
   ckks_ctx* ctx = b->ctx;
   const size_t nl = b->lanes.size();
@@ -80,8 +110,9 @@ int issue_all(ckks_batch* b) {
   if (e != cudaSuccess) return cuda_fail(ctx, e, "fork");
   for (size_t l = 1; l < nl; ++l)
     if ((e = cudaStreamWaitEvent(b->lanes[l]->stream, b->events[0], 0)) != cudaSuccess) return cuda_fail(ctx, e, "fork");
+  const std::vector<int> lane_of = assign_lanes(b);
   for (size_t i = 0; i < b->ops.size(); ++i) {
-    ckks_ctx* lane = b->lanes[i % nl];
+    ckks_ctx* lane = b->lanes[lane_of[i]];
     const int rc = issue_one(lane, b->ops[i]);
     if (rc != CKKS_OK) {
       if (lane != ctx) ctx->err = lane->err;
