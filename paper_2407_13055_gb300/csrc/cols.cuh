@@ -501,12 +501,22 @@ static bool with_shape(const ColShape& s, F f) {
 // 245.3 -> 235.7 by the rescale shape (level 3: 97.9 -> 83.6, 88.6; 108.9 ->
 // 107.3); at K <= 16 these run only below tensor_work (there 8 slices win: level
 // 1, dnum = 3, HRot 40.3 -> 37.9); N = 2^12: 16.7 -> 16.3 (HRot, dnum = 1).
+// Above 16 sources two targets at a time halve the reads of the sources' tile;
+// a ModUp or rescaling of few products (work, as in tensor_work) does better
+// with more blocks. Levels 3, 10, 20, 39 of dnum = 1, one target -> two: HRot by the
+// ModUp shape 75.8 -> 76.6, 98.4 -> 97.3, 132.5 -> 129.3, 194.6 -> 186.8, by the
+// ModDown shape 75.9 -> 75.3, 98.5 -> 97.4, 132.3 -> 129.0, 194.6 -> 188.0; HMult +
+// rescale 87.0 -> 86.7, 108.9 -> 106.6, 145.0 -> 140.8, 216.0 -> 209.4 (level 1
+// 78.8 -> 80.0).
 template <class G>
-static ColShape default_shape(ColKernel k, int K) {
+static ColShape default_shape(ColKernel k, int K, int work = 1 << 30) {
   if (G::W == 16) return ColShape{8, 4, 1, 1};
   if (G::W == 64) return ColShape{4, 8, k == CK_MODUP ? 1 : 2, 1};
-  if (k == CK_MODUP) return K > kTcMaxSources ? ColShape{8, 4, 2, 1} : ColShape{4, 8, 1, 1};
-  return k == CK_MODDOWN && K > kTcMaxSources ? ColShape{8, 4, 1, 1} : ColShape{8, 8, 1, 1};
+  if (K > kTcMaxSources) {
+    if (k == CK_MODUP) return work >= 400 ? ColShape{8, 8, 1, 2} : ColShape{8, 4, 2, 1};
+    return k == CK_MODDOWN || work >= 200 ? ColShape{8, 4, 1, 2} : ColShape{8, 8, 1, 1};
+  }
+  return k == CK_MODUP ? ColShape{4, 8, 1, 1} : ColShape{8, 8, 1, 1};
 }
 
 // A shape is launchable when the tile width divides the row, a slice is a
@@ -543,7 +553,8 @@ static ColShape pick_shape(const Scratch& sc, ColKernel k, int tix, int K, int w
     const ColShape s = sc.tune->get(k, tix);
     if (s.valid() && shape_ok<G>(s)) return s;
   }
-  return G::W == 1024 && K <= kTcMaxSources && work >= tensor_work(k) ? ColShape{8, 4, 1, 16} : default_shape<G>(k, K);
+  return G::W == 1024 && K <= kTcMaxSources && work >= tensor_work(k) ? ColShape{8, 4, 1, 16}
+                                                                                       : default_shape<G>(k, K, work);
 }
 
 // Whether a shape runs on the tensor cores for a conversion of K sources.
