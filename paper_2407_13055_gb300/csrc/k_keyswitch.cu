@@ -750,7 +750,9 @@ static void moddown_rescale_tail(const DevParams& dp, const Scratch& sc, const K
   prof_mark(sc, st, P_MODDOWN_IN_ROWS);
   launch_rs_cols_fused<G>(dp, n, sc, T3, pick_shape<G>(sc, CK_RS_FUSED, a.tix, alpha + 1, 2 * (alpha + 1) * top), st);
   prof_mark(sc, st, P_RS_COLS);
-  launch_rows_fwd<G>(dp, T3, EpiRsOut{a, A, a_stride}, 2 * top, LimbMap{nullptr, 0, top, top, dp.L}, st);
+  LimbMap out_map{nullptr, 0, top, top, dp.L};
+  out_map.pairs = top;  // both outputs of a limb read its inputs b1 and b2
+  launch_rows_fwd<G>(dp, T3, EpiRsOut{a, A, a_stride}, 2 * top, out_map, st);
   prof_mark(sc, st, P_RS_ROWS);
 }
 
