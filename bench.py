@@ -149,10 +149,10 @@ def multiply_costs(rates):
 # sources (kernel_sources) differs, the figures are stale and the bench
 # reports null.
 NCU_TRAFFIC = {
-    "sources_sha1": "7752ec4617116707750c987e104ac7492e35ba55",
-    "bytes_per_launch": {"modup_cols": 10.58e6, "keymult": 135.59e6, "modup_rows": 60.32e6,
-                         "moddown_in_rows": 15.76e6, "moddown_cols": 7.40e6, "moddown_rows": 74.29e6,
-                         "rescale_cols": 7.95e6, "rescale_rows": 118.13e6, "ks_in_rows": 37.31e6},
+    "sources_sha1": "54afaf30d200be28e38e9f7e78c16c200ba3d42b",
+    "bytes_per_launch": {"modup_cols": 10.65e6, "keymult": 134.73e6, "modup_rows": 60.44e6,
+                         "moddown_in_rows": 15.76e6, "moddown_cols": 7.45e6, "moddown_rows": 75.32e6,
+                         "rescale_cols": 7.99e6, "rescale_rows": 107.18e6, "ks_in_rows": 37.30e6},
 }
 
 
@@ -762,13 +762,13 @@ def e2e_leg(K, ctx, lanes, streams, stream, cts, rk, gk, n_lanes, slots, steps, 
     return e2e
 
 
-def tensor_core_leg(K, ctx, ops, n_lanes, stream, steps, warmup, cuda_core_ops_s, shape=(4, 8, 1, 16)):
+def tensor_core_leg(K, ctx, ops, n_lanes, stream, steps, warmup, tensor_core_ops_s, shape=(4, 8, 1, 1)):
     """The headline's operations (one CUDA graph per step over n_lanes lanes)
-    with the BConv of every column kernel on the tensor cores (tcgen05, exact
-    fp16 byte planes; launch shape tc, sl, z, targets per chunk) instead of
-    CUDA cores, on the same context and inputs; the tuned shapes are put back
-    afterwards. Returns ops/s beside the CUDA-core figure and the operations'
-    HBM fraction."""
+    with the BConv of every column kernel on CUDA cores (launch shape tc, sl,
+    z, targets at a time) instead of the tensor cores (tcgen05, exact fp16 byte
+    planes; the rule's choice at these sizes), on the same context and inputs;
+    the tuned shapes are put back afterwards. Returns ops/s beside the
+    headline's figure and the operations' HBM fraction."""
     import torch
     kernels = (K.CKKS_COL_MODUP, K.CKKS_COL_MODDOWN, K.CKKS_COL_RS_FUSED)
     saved = {k: K.ckks_tune_get(ctx, k, LEVEL) for k in kernels}
@@ -795,12 +795,12 @@ def tensor_core_leg(K, ctx, ops, n_lanes, stream, steps, warmup, cuda_core_ops_s
     ops_s = len(ops) * steps / (ms / 1e3)
     mean_bytes = (algorithmic_bytes()[0] + algorithmic_bytes()[1]) / 2
     peaks, kind = measured_peaks()
-    return {"ops_s": ops_s, "cuda_core_ops_s": cuda_core_ops_s, "col_shape": list(shape),
-            "op_frac_of_hbm": ops_s * mean_bytes / 1e9 / peaks["hbm_gbs"],
-            "cuda_core_op_frac_of_hbm": cuda_core_ops_s * mean_bytes / 1e9 / peaks["hbm_gbs"],
+    return {"ops_s": tensor_core_ops_s, "cuda_core_ops_s": ops_s, "cuda_core_col_shape": list(shape),
+            "op_frac_of_hbm": tensor_core_ops_s * mean_bytes / 1e9 / peaks["hbm_gbs"],
+            "cuda_core_op_frac_of_hbm": ops_s * mean_bytes / 1e9 / peaks["hbm_gbs"],
             "note": f"{steps} graph replays of the same {len(ops)} operations, every column kernel's BConv on "
-                    f"the tensor cores (shape {shape}), against the headline's tuned CUDA-core shapes; "
-                    f"HBM fraction of {kind} hbm_gbs"}
+                    f"CUDA cores (shape {shape}), against the headline's shapes (the tensor cores, unless the "
+                    f"tuner chose otherwise); HBM fraction of {kind} hbm_gbs"}
 
 
 def fusion_ablation(K, ctx, sk, rk, gk, stream, levels=(L - 1, 20, 1), reps=15, pdl=True):
@@ -1434,8 +1434,7 @@ def main():
                     help="tc,sl,z,tp: use this launch shape for the three column kernels at every level instead "
                          "of the tuner's (tp 8/16: tensor-core BConv)")
     ap.add_argument("--row-passes", type=int, default=None, choices=[2, 3, 4, 5, 6],
-                    help="N=2^16 row-phase form instead of the tuner's (4, 5: forward rows staged by bulk copies; "
-                         "6: twiddles in shared memory)")
+                    help="N=2^16 row-phase form instead of the tuner's (register passes; 4 to 6 run as 3)")
     ap.add_argument("--e2e-slots", type=int, default=2,
                     help="buffer slots per lane of the end-to-end upload / compute / export pipeline")
     ap.add_argument("--e2e-priority", choices=["high", "normal"], default="high",

@@ -234,7 +234,7 @@ enum ProfId {
   P_MODDOWN_IN_ROWS,  // iNTT row phase of the P limbs
   P_MODDOWN_COLS,     // iNTT cols, BConv P -> Q, NTT cols
   P_MODDOWN_ROWS,     // NTT row phase of the converted limbs
-  P_KS_EPILOGUE,      // (acc - z) P^-1 + d0/d1 or phi(b) (streaming)
+  P_KS_EPILOGUE,      // linear transform without a rotated term (streaming)
   P_RS_IN_ROWS,       // rescale: iNTT rows of the top limb
   P_RS_COLS,          // rescale: iNTT cols, reduce, NTT cols
   P_RS_ROWS,          // rescale: NTT rows
@@ -313,7 +313,7 @@ struct Scratch {
   uint32_t* S;  // row-phase iNTT outputs (ModUp input, ModDown P-limbs)
   uint32_t* T;  // column-phase outputs [dnum][L + alpha][N] (ModUp), then [2][L][N] (ModDown)
   uint32_t* A;  // accumulators [2][n + alpha][N]
-  uint32_t* U;  // centered coefficients of the fused ModDown + rescale [2][alpha + 1][N]; staged HMult output
+  uint32_t* U;  // HMult's output before a rational rescale (a windowed context)
   Prof* prof;   // optional stage timing (null or off: no events)
   const Tuning* tune = nullptr;  // tuned column-kernel shapes (null: default rule)
 };
