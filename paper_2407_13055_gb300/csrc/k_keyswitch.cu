@@ -247,19 +247,20 @@ static void launch_keymult(int digits, dim3 g, int th, cudaStream_t st, const De
 //
 // Sums are kept in 64 bits below 2^32 q (fold64): per term the digits' products
 // fold, one Montgomery reduction (the key's factor cancels it), times the
-// plaintext, fold. Digits one after the other at 64 registers and four blocks
-// per SM (3 or 5 blocks: 1 % and 5 % slower), each load a full quad. Bound by
+// plaintext, fold. Digits one after the other at 56 registers and nine blocks
+// per SM (7: 1 % slower; blocks of 256, 3 to 5 per SM: 1 to 7 %), each load a full
+// quad. Bound by
 // the keys: 16 terms at level 33 stream 1.13 GB of keys and 0.2 GB of
 // plaintexts, 199 us at the copy rate. Measured there: 261 us, and 52 us for
-// the other terms after the ModDown, -> 244 us for both; the operation 391.7 ->
-// 329 us.
+// the other terms after the ModDown, -> 240 us for both; the operation 391.7 ->
+// 325 us.
 __device__ __forceinline__ uint32_t reduce_sum(uint64_t s, const PrimeConst& P) {  // s < 2^32 q -> [0, q)
   const uint32_t t = csub(csub(redc64(s, P.q, P.m), P.q), P.q);                    // s 2^-32
   return fix_signed(smr((int64_t)t * P.r2c, P.q, P.m), P.q);
 }
 
 template <int D>
-__global__ void __launch_bounds__(256, 4) k_lt_keymult(DevParams dp, KsArgs a, const __grid_constant__ LtArgs lt,
+__global__ void __launch_bounds__(128, 9) k_lt_keymult(DevParams dp, KsArgs a, const __grid_constant__ LtArgs lt,
                                                     const uint32_t* T, uint32_t* A) {
   pdl_wait();
   pdl_trigger();
@@ -708,10 +709,13 @@ static int groups_for(int blocks_per_group, int max_groups, int sms) {
   return g < 1 ? 1 : g;
 }
 
-// Streaming grid: four positions per thread.
+// Streaming grid: four positions per thread. Blocks of 128 threads end and start
+// more evenly than of 256 (HMult + rescale level 39 137.3 -> 136.5 us, the 25-30
+// system's level 6 58.4 -> 57.8, linear transform 329.4 -> 326.4); of 64 they start too
+// slowly (HMult level 20 78.4 -> 83.0).
 static void stream_grid(int log_n, int limbs, dim3& grid, int& threads) {
   const int quads = (1 << log_n) / 4;
-  threads = quads < 256 ? quads : 256;
+  threads = quads < 128 ? quads : 128;
   grid = dim3(quads / threads, limbs);
 }
 
