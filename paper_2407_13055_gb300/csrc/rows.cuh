@@ -297,9 +297,12 @@ __global__ void __launch_bounds__(G::RT) k_rows_inv_t(DevParams dp, Src src, uin
 // runs per access of a warp: with the C layout's 16 consecutive words per
 // thread each 16-byte access touched 32 sectors and used half of each.
 //
-// Launch bounds of 12 blocks of 2 warps per SM (80 registers): 24 resident
+// Launch bounds, forward: 12 blocks of 2 warps per SM (80 registers), 24 resident
 // warps, against 16 for the two-pass form at 128 registers (14 blocks: 17.6 us
-// for the ModUp rows of two-row blocks, 10: 18.6).
+// for the ModUp rows of two-row blocks, 10: 18.6; HRot level 39 118.8 us at 12,
+// 121.0 at 10). Inverse: 10 blocks (96 registers), whose sources keep more loads
+// in flight (HMult + rescale level 39 136.5 us at 12, 134.9 at 10, 9 and 8; level 20
+// 78.3, 76.8; the 25-30 system's level 6 57.9, 56.6).
 //
 // Bound and figures (ModUp rows at the top level, 40 primes, dnum = 3, 122
 // limbs, launched back to back): 24.4 us with the XOR swizzle, table-order
@@ -490,7 +493,7 @@ __global__ void __launch_bounds__(64 * kRow3Rows, 12 / kRow3Rows)
 }
 
 template <class G, class Src>
-__global__ void __launch_bounds__(64 * kRow3Rows, 12 / kRow3Rows)
+__global__ void __launch_bounds__(64 * kRow3Rows, 10 / kRow3Rows)
     k_rows3_inv_t(DevParams dp, Src src, uint32_t* dst, LimbMap map, int dst_compact) {
   static_assert(G::W == 1024, "three-pass rows are for W = 1024");
   __shared__ __align__(16) uint32_t buf[kRow3Rows][kRow3Words];
