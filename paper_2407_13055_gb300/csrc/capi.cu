@@ -1478,7 +1478,9 @@ int ckks_step_moddown(ckks_ctx* ctx, const uint32_t* acc, int n_q, uint32_t* out
   int rc = cuda_check(ctx, cudaMemcpyAsync(dcan.p, acc, in_limbs * lw * 4, cudaMemcpyHostToDevice, ctx->stream), "upload");
   if (rc) return rc;
   launch_permute(ctx->dp, dcan.as<uint32_t>(), din.as<uint32_t>(), (int)in_limbs, true, ctx->stream);
-  launch_moddown(ctx->dp, ctx->sc, din.as<uint32_t>(), n_q, dout.as<uint32_t>(), ctx->stream);
+  // the first n_q primes need not be a level's window (level windows)
+  const bool level = n_q <= ctx->n_levels() && ctx->lvl_base(n_q - 1) == 0 && ctx->lvl_n(n_q - 1) == n_q;
+  launch_moddown(ctx->dp, ctx->sc, din.as<uint32_t>(), n_q, level ? n_q : 0, dout.as<uint32_t>(), ctx->stream);
   launch_permute(ctx->dp, dout.as<uint32_t>(), dres.as<uint32_t>(), (int)out_limbs, false, ctx->stream);
   rc = cuda_check(ctx, cudaMemcpyAsync(out, dres.p, out_limbs * lw * 4, cudaMemcpyDeviceToHost, ctx->stream), "download");
   return rc ? rc : finish(ctx, "moddown step");

@@ -582,7 +582,8 @@ void launch_modup_cols(const DevParams& dp, int n, int base, int tix, int digits
 template <class G>
 void launch_moddown_cols(const DevParams& dp, int n, int base, int tix, const Scratch& sc, const ColShape& s0,
                          cudaStream_t st) {
-  if (use_tc<G>(dp, s0, dp.alpha)) return launch_moddown_tc<G>(dp, n, base, tix, sc, st);
+  // tix 0: the window is no level's, whose image and work division the tensor-core form takes
+  if (tix > 0 && use_tc<G>(dp, s0, dp.alpha)) return launch_moddown_tc<G>(dp, n, base, tix, sc, st);
   const ColShape s = is_tc_shape(s0) ? default_shape<G>(CK_MODDOWN, dp.alpha) : s0;
   with_shape(s, [&](auto tc, auto sl, auto tp) {
     constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, TP = decltype(tp)::value;

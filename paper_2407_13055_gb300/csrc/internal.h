@@ -412,7 +412,9 @@ void launch_linear_transform(const DevParams& dp, const Scratch& sc, const KsArg
                              cudaStream_t st);
 void launch_rational_rescale(const DevParams& dp, const Scratch& sc, const RrArgs& r, const uint32_t* in,
                              size_t sin, uint32_t* out, size_t sout, cudaStream_t st);
-void launch_moddown(const DevParams& dp, const Scratch& sc, const uint32_t* acc, int n, uint32_t* out,
+// tix: the level whose window is the first n primes, plus one; 0 if no level
+// has that window (then nothing made per level is used).
+void launch_moddown(const DevParams& dp, const Scratch& sc, const uint32_t* acc, int n, int tix, uint32_t* out,
                     cudaStream_t st);
 // Rescale: in [2][n][N] (stride sin) -> out [2][n-1][N] (stride sout).
 // tensor: the column phase may run in its tensor-core form, whose first launch

@@ -1189,11 +1189,11 @@ void launch_rational_rescale(const DevParams& dp, const Scratch& sc, const RrArg
   });
 }
 
-void launch_moddown(const DevParams& dp, const Scratch& sc, const uint32_t* acc, int n, uint32_t* out,
+void launch_moddown(const DevParams& dp, const Scratch& sc, const uint32_t* acc, int n, int tix, uint32_t* out,
                     cudaStream_t st) {
   KsArgs a{};
   a.n = n;
-  a.tix = n;
+  a.tix = tix;
   a.out = out;
   a.out_stride = (size_t)n << dp.log_n;
   a.extra = 0;
