@@ -570,6 +570,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // every product is done before A is written again
     gc += np / 4;
     wait(b_full((gc - 1) & 1), ((gc - 1) >> 1) & 1);
+    tc::fence_after_sync();  // a warpgroup without a target in the last group has not ordered itself behind it
     ++it_no;
     seg = nseg;
     have = more;
