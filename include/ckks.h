@@ -484,8 +484,9 @@ int ckks_set_launch_flags(ckks_ctx* ctx, int flags);
  * usable. The limit applies to kernels enqueued after the call; a clone
  * inherits the parent's limit when it is created. The tensor-core column
  * kernels wait for their own copies and products only, which end in
- * microseconds; they give up after at least 2^24 cycles whatever the limit.
- * CKKS_EINVAL if cycles < 1.
+ * microseconds: where the library chose them (by rule or by ckks_tune) they
+ * give up after at least 2^24 cycles whatever the limit, where ckks_tune_set
+ * did, after the limit as it is. CKKS_EINVAL if cycles < 1.
  * (Not from the paper: a guard of this implementation's asynchronous
  * kernels.) */
 int ckks_set_wait_limit(ckks_ctx* ctx, long long cycles);

@@ -567,7 +567,7 @@ static bool use_tc(const DevParams& dp, const ColShape& s, int K) {
 template <class G>
 void launch_modup_cols(const DevParams& dp, int n, int base, int tix, int digits, const Scratch& sc,
                        const ColShape& s0, cudaStream_t st) {
-  if (use_tc<G>(dp, s0, dp.alpha)) return launch_modup_tc<G>(dp, n, base, tix, digits, sc, st);
+  if (use_tc<G>(dp, s0, dp.alpha)) return launch_modup_tc<G>(dp, n, base, tix, digits, sc, s0, st);
   const ColShape s = is_tc_shape(s0) ? default_shape<G>(CK_MODUP, dp.alpha) : s0;
   with_shape(s, [&](auto tc, auto sl, auto tp) {
     constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, TP = decltype(tp)::value;
@@ -583,7 +583,7 @@ template <class G>
 void launch_moddown_cols(const DevParams& dp, int n, int base, int tix, const Scratch& sc, const ColShape& s0,
                          cudaStream_t st) {
   // tix 0: the window is no level's, whose image and work division the tensor-core form takes
-  if (tix > 0 && use_tc<G>(dp, s0, dp.alpha)) return launch_moddown_tc<G>(dp, n, base, tix, sc, st);
+  if (tix > 0 && use_tc<G>(dp, s0, dp.alpha)) return launch_moddown_tc<G>(dp, n, base, tix, sc, s0, st);
   const ColShape s = is_tc_shape(s0) ? default_shape<G>(CK_MODDOWN, dp.alpha) : s0;
   with_shape(s, [&](auto tc, auto sl, auto tp) {
     constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, TP = decltype(tp)::value;
@@ -598,7 +598,7 @@ void launch_moddown_cols(const DevParams& dp, int n, int base, int tix, const Sc
 template <class G>
 void launch_rs_cols_fused(const DevParams& dp, int n, const Scratch& sc, uint32_t* T3, const ColShape& s0,
                           cudaStream_t st) {
-  if (use_tc<G>(dp, s0, dp.alpha + 1)) return launch_rs_fused_tc<G>(dp, n, sc, T3, st);
+  if (use_tc<G>(dp, s0, dp.alpha + 1)) return launch_rs_fused_tc<G>(dp, n, sc, T3, s0, st);
   const ColShape s = is_tc_shape(s0) ? default_shape<G>(CK_RS_FUSED, dp.alpha + 1) : s0;
   with_shape(s, [&](auto tc, auto sl, auto tp) {
     constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, TP = decltype(tp)::value;
@@ -612,7 +612,7 @@ void launch_rs_cols_fused(const DevParams& dp, int n, const Scratch& sc, uint32_
 
 template <class G>
 void launch_mm_cols(const DevParams& dp, const MmArgs& m, const Scratch& sc, const ColShape& s0, cudaStream_t st) {
-  if (m.img >= 0 && use_tc<G>(dp, s0, m.K)) return launch_mm_tc<G>(dp, m, sc, st);
+  if (m.img >= 0 && use_tc<G>(dp, s0, m.K)) return launch_mm_tc<G>(dp, m, sc, s0, st);
   const ColShape s = is_tc_shape(s0) ? default_shape<G>(CK_RS_FUSED, m.K) : s0;
   with_shape(s, [&](auto tc, auto sl, auto tp) {
     constexpr int TC = decltype(tc)::value, SL = decltype(sl)::value, TP = decltype(tp)::value;

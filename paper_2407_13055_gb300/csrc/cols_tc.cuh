@@ -40,9 +40,10 @@
 // 3000 cycles) and the first product of each segment.
 //
 // Every mbarrier wait is bounded. When one expires the block records the
-// timeout in dp.status and skips all further waits: its results are undefined
-// but every access stays in bounds, and it ends after draining (bounded) its
-// own copies and products; the host reports CKKS_ETIMEOUT at the next
+// timeout in dp.status, skips all further waits and starts no further copy (a
+// segment buffer's barrier takes one copy group at a time): its results are
+// undefined but no address depends on them, and it ends after its own products
+// and copies (bounded again); the host reports CKKS_ETIMEOUT at the next
 // synchronizing call.
 #pragma once
 #include "tc.cuh"
@@ -54,8 +55,8 @@ constexpr int kTcMaxSources = 16;
 // Targets per segment (shared-memory room for their planes and twiddles).
 constexpr int kTcCap = 56;
 // Cycles any wait on a block's own copies and products may take at least
-// (about 8 ms): they end in microseconds, whatever dp.wait_limit asks for
-// waits on the host.
+// (about 8 ms) where the shape was not set by hand: they end in microseconds,
+// whatever dp.wait_limit asks for waits on the host.
 constexpr long long kTcWaitFloor = 1ll << 24;
 constexpr long long kTcDrainLimit = 1ll << 32;
 
@@ -141,7 +142,7 @@ inline TcLayout tc_layout(int cap, int kr) {
   s.trec = s.srec + kTcMaxSources * kTcRecBytes;
   s.seg_bytes = s.trec + (uint32_t)cap * kTcRecBytes;
   s.bar = s.seg + 2 * s.seg_bytes;
-  s.total = s.bar + 7 * 8 + 8;
+  s.total = s.bar + 8 * 8 + 8;
   return s;
 }
 
@@ -265,14 +266,20 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   auto b_ld = [&](int i) { return bars + 8u * i; };
   auto b_full = [&](int i) { return bars + 16u + 8u * i; };
   auto b_empty = [&](int i) { return bars + 32u + 8u * i; };
-  const uint32_t b_a = bars + 48u;
-  volatile uint32_t* slot = reinterpret_cast<volatile uint32_t*>(sm + lay.bar + 56);
-  volatile uint32_t* flag = reinterpret_cast<volatile uint32_t*>(sm + lay.bar + 60);
-  const long long limit = dp.wait_limit > kTcWaitFloor ? dp.wait_limit : kTcWaitFloor;
+  const uint32_t b_a = bars + 48u, b_done = bars + 56u;
+  volatile uint32_t* slot = reinterpret_cast<volatile uint32_t*>(sm + lay.bar + 64);
+  volatile uint32_t* flag = reinterpret_cast<volatile uint32_t*>(sm + lay.bar + 68);
+  const long long limit = dp.wait_limit;
   auto wait = [&](uint32_t bar, uint32_t parity) {
-    if (tc::mbar_try(bar, parity)) return;
-    if (*flag) return;
-    if (!tc::mbar_wait(bar, parity, limit)) {
+    if (!tc::mbar_try(bar, parity) && !*flag && !tc::mbar_wait(bar, parity, limit)) {
+      *flag = 1;
+      tc::report_timeout(dp.status);
+    }
+  };
+  // The products' wait for the sources, which takes a block's longest: a limit
+  // below kPollLimit expires here, before the blocking try.
+  auto wait_sources = [&](uint32_t parity) {
+    if (!*flag && !tc::mbar_wait(b_a, parity, limit)) {
       *flag = 1;
       tc::report_timeout(dp.status);
     }
@@ -298,6 +305,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           tc::mbar_init(b_empty(i), 16);  // the warps of four targets
         }
         tc::mbar_init(b_a, kTcWarpgroups * 4);
+        tc::mbar_init(b_done, kTcMmaWarps);
         tc::mbar_init_fence();
         *flag = 0;
       }
@@ -338,7 +346,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    if (have && mw == 0 && lane == 0) load(seg, 0);
+    int loads = 0;  // of the lane that loads
+    if (have && mw == 0 && lane == 0) {
+      load(seg, 0);
+      ++loads;
+    }
     __syncwarp();
     const uint32_t tmem = *slot;
     int it_no = 0, gc = 0, a_no = 0;
@@ -350,11 +362,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       const uint32_t sbo = (uint32_t)kr * 16u, gb = (uint32_t)kr * 32u;
       uint32_t b0 = tc::smem_u32(sm + lay.seg + (it_no & 1) * lay.seg_bytes);
       wait(b_ld(it_no & 1), (it_no >> 1) & 1);
-      wait(b_a, a_no & 1);
+      wait_sources(a_no & 1);
       ++a_no;
       tc::fence_after_sync();
-      // every warpgroup is past the previous segment: its buffer is free
-      if (more && mw == 0 && lane == 0) load(nx, (it_no + 1) & 1);
+      // every warpgroup is past the previous segment: its buffer is free (with
+      // the flag down, the waits so far, that for the buffer's last copies
+      // among them, ended by completion)
+      if (more && mw == 0 && lane == 0 && !*flag) {
+        load(nx, (it_no + 1) & 1);
+        ++loads;
+      }
       __syncwarp();
       auto product = [&]() {
         if (gc >= 2) {
@@ -375,7 +392,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       };
       if constexpr (TOP) {
         product();
-        wait(b_a, a_no & 1);
+        wait_sources(a_no & 1);
         ++a_no;
         tc::fence_after_sync();
       }
@@ -385,10 +402,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       seg = nx;
       have = more;
     }
-    // drain: products and copies still in flight after a timeout
-    if (*flag && lane == 0) {
-      for (int u = gc < 2 ? 0 : gc - 2; u < gc; ++u) tc::mbar_wait(b_full(u & 1), (u >> 1) & 1, kTcDrainLimit);
-      for (int u = it_no < 2 ? 0 : it_no - 2; u < it_no; ++u) tc::mbar_wait(b_ld(u & 1), (u >> 1) & 1, kTcDrainLimit);
+    // the block ends after all its products and copies, after a timeout too
+    tc::commit(b_done);
+    if (lane == 0) {
+      tc::mbar_wait(b_done, 0, kTcDrainLimit);
+      for (int u = loads < 2 ? 0 : loads - 2; u < loads; ++u) tc::mbar_wait(b_ld(u & 1), (u >> 1) & 1, kTcDrainLimit);
     }
     __syncwarp();
     tc::fence_before_sync();
@@ -583,9 +601,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // Launch
 // ---------------------------------------------------------------------------
 
+// exact_limit: dp.wait_limit as it is, without the floor (a shape set by hand).
 template <class G, bool TOP>
-void launch_cols_tc(const DevParams& dp, const TcJob& job, int groups, int2 plan, cudaStream_t st) {
+void launch_cols_tc(const DevParams& dp0, const TcJob& job, int groups, int2 plan, bool exact_limit, cudaStream_t st) {
   if constexpr (G::H == 64) {
+    DevParams dp = dp0;
+    if (!exact_limit) dp.wait_limit = std::max(dp.wait_limit, kTcWaitFloor);
     int kr = 16, cap = 4;
     for (int g = 0; g < groups; ++g) {
       kr = std::max(kr, tc_kr(job.g[g].K));
@@ -602,17 +623,17 @@ void launch_cols_tc(const DevParams& dp, const TcJob& job, int groups, int2 plan
 }
 
 // Compiled once, in k_cols_tc.cu.
-extern template void launch_cols_tc<Geo<8, 32>, false>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
-extern template void launch_cols_tc<Geo<8, 32>, true>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
-extern template void launch_cols_tc<Geo<8, 8>, false>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
-extern template void launch_cols_tc<Geo<8, 8>, true>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
-extern template void launch_cols_tc<Geo<4, 4>, false>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
-extern template void launch_cols_tc<Geo<4, 4>, true>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
+extern template void launch_cols_tc<Geo<8, 32>, false>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
+extern template void launch_cols_tc<Geo<8, 32>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
+extern template void launch_cols_tc<Geo<8, 8>, false>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
+extern template void launch_cols_tc<Geo<8, 8>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
+extern template void launch_cols_tc<Geo<4, 4>, false>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
+extern template void launch_cols_tc<Geo<4, 4>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
 
 // ModUp of the level's digits: each to every other prime of the extended basis.
 template <class G>
 static void launch_modup_tc(const DevParams& dp, int n, int base, int tix, int digits, const Scratch& sc,
-                            cudaStream_t st) {
+                            const ColShape& s, cudaStream_t st) {
   TcJob job{n, base, {}};
   for (int j = 0; j < digits; ++j) {
     const int g = base / dp.alpha + j;
@@ -623,38 +644,40 @@ static void launch_modup_tc(const DevParams& dp, int n, int base, int tix, int d
                        sc.T + ((size_t)j * (n + dp.alpha) << dp.log_n), hi - lo, n + dp.alpha - (hi - lo), base + lo, lo,
                        hi - lo};
   }
-  launch_cols_tc<G, false>(dp, job, digits, dp.ks.h_up_plan[tix], st);
+  launch_cols_tc<G, false>(dp, job, digits, dp.ks.h_up_plan[tix], s.by_hand, st);
 }
 
 // ModDown of both polynomials to the window.
 template <class G>
-static void launch_moddown_tc(const DevParams& dp, int n, int base, int tix, const Scratch& sc, cudaStream_t st) {
+static void launch_moddown_tc(const DevParams& dp, int n, int base, int tix, const Scratch& sc, const ColShape& s,
+                              cudaStream_t st) {
   TcJob job{n, base, {}};
   for (int u = 0; u < 2; ++u)
     job.g[u] = TcGroup{sc.S + ((size_t)u * dp.alpha << dp.log_n), dp.ks.dn_cin, dp.ks.tc_img + dp.ks.h_dn_img[tix].x,
                        nullptr, nullptr, sc.T + ((size_t)u * n << dp.log_n), dp.alpha, n, dp.L, n, 0};
-  launch_cols_tc<G, false>(dp, job, 2, dp.ks.h_dn_plan[tix], st);
+  launch_cols_tc<G, false>(dp, job, 2, dp.ks.h_dn_plan[tix], s.by_hand, st);
 }
 
 // ModDown fused with rescaling by the top prime.
 template <class G>
-static void launch_rs_fused_tc(const DevParams& dp, int n, const Scratch& sc, uint32_t* T3, cudaStream_t st) {
+static void launch_rs_fused_tc(const DevParams& dp, int n, const Scratch& sc, uint32_t* T3, const ColShape& s,
+                               cudaStream_t st) {
   TcJob job{n - 1, 0, {}};
   for (int u = 0; u < 2; ++u)
     job.g[u] = TcGroup{sc.S + ((size_t)u * dp.alpha << dp.log_n), dp.ks.dn_cin, dp.ks.tc_img + dp.ks.h_rs_img[n].x,
                        nullptr, sc.S + ((size_t)(2 * dp.alpha + u) << dp.log_n),
                        T3 + ((size_t)u * (n - 1) << dp.log_n), dp.alpha + 1, n - 1, dp.L, n, 0};
-  launch_cols_tc<G, true>(dp, job, 2, dp.ks.h_rs_plan[n], st);
+  launch_cols_tc<G, true>(dp, job, 2, dp.ks.h_rs_plan[n], s.by_hand, st);
 }
 
 // ModDown merged into the rescaling (Sec. 6).
 template <class G>
-static void launch_mm_tc(const DevParams& dp, const MmArgs& m, const Scratch& sc, cudaStream_t st) {
+static void launch_mm_tc(const DevParams& dp, const MmArgs& m, const Scratch& sc, const ColShape& s, cudaStream_t st) {
   TcJob job{m.n1, m.s1, {}};
   for (int u = 0; u < 2; ++u)
     job.g[u] = TcGroup{sc.S + ((size_t)u * m.K << dp.log_n), m.cin, dp.ks.tc_img + m.img, m.rows, nullptr,
                        sc.T + ((size_t)u * m.n1 << dp.log_n), m.K, m.n1, 0, m.n1, 0};
-  launch_cols_tc<G, false>(dp, job, 2, m.plan, st);
+  launch_cols_tc<G, false>(dp, job, 2, m.plan, s.by_hand, st);
 }
 
 // Rescaling by the top prime q_(n-1): its limb of both polynomials (S = [2])
@@ -666,7 +689,7 @@ static void launch_rescale_tc(const DevParams& dp, int n, const Scratch& sc, cud
     job.g[u] = TcGroup{sc.S + ((size_t)u << dp.log_n), reinterpret_cast<const uint2*>(&dp.pc[n - 1].ninv),
                        dp.ks.tc_img + dp.ks.one_img, nullptr, nullptr, sc.T + ((size_t)u * (n - 1) << dp.log_n), 1,
                        n - 1, n - 1, n, 0};
-  launch_cols_tc<G, false>(dp, job, 2, dp.ks.h_one_plan[n], st);
+  launch_cols_tc<G, false>(dp, job, 2, dp.ks.h_one_plan[n], false, st);
 }
 
 // Rational rescaling: the dropped limbs (S = [K][2]) to the new window.
@@ -676,7 +699,7 @@ static void launch_rr_tc(const DevParams& dp, const RrArgs& r, const Scratch& sc
   for (int u = 0; u < 2; ++u)
     job.g[u] = TcGroup{sc.S + ((size_t)u << dp.log_n), r.cin, dp.ks.tc_img + r.img, r.drop, nullptr,
                        sc.T + ((size_t)u * r.n1 << dp.log_n), r.K, r.n1, 0, r.n1, 0, 2};
-  launch_cols_tc<G, false>(dp, job, 2, r.plan, st);
+  launch_cols_tc<G, false>(dp, job, 2, r.plan, false, st);
 }
 
 // Tensor-core launch shapes: tp = 8 or 16 with the (tc, sl) pairs below and

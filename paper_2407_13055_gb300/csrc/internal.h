@@ -268,6 +268,7 @@ enum ColKernel { CK_MODUP = 0, CK_MODDOWN = 1, CK_RS_FUSED = 2, CK_ROWS = 3, CK_
 
 struct ColShape {
   int tc = 0, sl = 0, z = 0, tp = 1;  // tp: conversion targets per pass (1 or 2)
+  bool by_hand = false;  // set by ckks_tune_set (the waits of a tensor-core shape keep the limit as it is)
   bool valid() const { return tc > 0; }
 };
 
@@ -290,6 +291,7 @@ struct Tuning {
       s.sl = (int)((v >> 8) & 0xff);
       s.z = (int)((v >> 16) & 0xff);
       s.tp = (int)((v >> 24) & 0xff);
+      s.by_hand = us[k * (max_n + 1) + n].load(std::memory_order_relaxed) == 0.f;  // no measured time
     }
     return s;
   }

@@ -3,11 +3,11 @@
 
 namespace ckks {
 
-template void launch_cols_tc<Geo<8, 32>, false>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
-template void launch_cols_tc<Geo<8, 32>, true>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
-template void launch_cols_tc<Geo<8, 8>, false>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
-template void launch_cols_tc<Geo<8, 8>, true>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
-template void launch_cols_tc<Geo<4, 4>, false>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
-template void launch_cols_tc<Geo<4, 4>, true>(const DevParams&, const TcJob&, int, int2, cudaStream_t);
+template void launch_cols_tc<Geo<8, 32>, false>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
+template void launch_cols_tc<Geo<8, 32>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
+template void launch_cols_tc<Geo<8, 8>, false>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
+template void launch_cols_tc<Geo<8, 8>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
+template void launch_cols_tc<Geo<4, 4>, false>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
+template void launch_cols_tc<Geo<4, 4>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
 
 }  // namespace ckks

@@ -137,14 +137,15 @@ __device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
 }
 
 // Bounded wait: true once the phase completed, false after `limit` SM clock
-// cycles without completion. Limits below 1024 cycles poll with the
+// cycles without completion. Limits below kPollLimit cycles poll with the
 // non-blocking test only (a blocking try may sleep past such a limit), so a
 // limit of a few cycles expires whenever the phase is still pending at the
 // call; longer limits let the hardware suspend the waiting warp.
+constexpr long long kPollLimit = 1024;
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long long limit) {
   if (mbar_test(mbar, parity)) return true;
   const long long t0 = clock64();
-  if (limit < 1024) {
+  if (limit < kPollLimit) {
     while (clock64() - t0 <= limit)
       if (mbar_test(mbar, parity)) return true;
     return false;
