@@ -8,13 +8,12 @@
 // parallel.
 #pragma once
 #include <algorithm>
-#include <map>
-#include <mutex>
 #include <type_traits>
 
 #include "geo.cuh"
 #include "internal.h"
 #include "pdl.cuh"
+#include "smem_limits.h"
 #include "tc.cuh"
 
 namespace ckks {
@@ -444,18 +443,16 @@ static size_t col_smem_bytes(int K) {
   return (size_t)K * (G::EC / 4) * CTL::CT * sizeof(int4) + (size_t)SL * CTL::BUF * sizeof(uint32_t);
 }
 
-// Raise a kernel's dynamic shared-memory limit once per process (and only
+// Raise a kernel's dynamic shared-memory limit once per device (and only
 // when a larger size is needed), so that steady-state launches and graph
-// captures issue no attribute calls.
+// captures issue no attribute calls. A failure is the launch's error.
 static void set_col_smem(const void* f, size_t bytes) {
-  static std::mutex mu;
-  static std::map<const void*, size_t> done;
-  std::lock_guard<std::mutex> lock(mu);
-  size_t& cur = done[f];
-  if (bytes > cur) {
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    cur = bytes;
-  }
+  static SmemLimits limits;
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess) return;
+  limits.at_least(device, f, bytes, [&] {
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+  });
 }
 
 // ---------------------------------------------------------------------------
