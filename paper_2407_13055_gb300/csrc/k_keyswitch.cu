@@ -137,10 +137,14 @@ __device__ __forceinline__ void ks_input4(const DevParams& dp, const KsArgs& a, 
 // them), the others come from the NTT'd ModUp output T[j][t]. All loads of a
 // thread are issued before any product so that one memory latency covers the
 // whole sum. A = [2][n + alpha][N]. With wait_dep the programmatic-dependent-
-// launch wait sits after the index arithmetic and before the first load.
-template <int D>
+// launch wait sits after the index arithmetic and before the first load. GATHER:
+// a.hoisted may be set. (The persistent kernel, whose operations are never
+// hoisted, holds every digit count's code; with the gather's registers in it
+// it spilled: 24 products at level 39 907 us instead of 517.)
+template <int D, bool GATHER>
 __device__ __forceinline__ void keymult_quad(const DevParams& dp, const KsArgs& a, const uint32_t* T, uint32_t* A,
                                              int t, uint32_t p0, int km_out, uint32_t* km_dst, bool wait_dep) {
+  const bool hoisted = GATHER && a.hoisted;
   const int n = a.n, alpha = dp.alpha, L = dp.L, ext = n + alpha, ext_top = L + alpha;
   const int id = prime_of(t, n, L, a.base);
   const int key_limb = id;  // keys cover every prime: limb = global prime index
@@ -160,7 +164,7 @@ __device__ __forceinline__ void keymult_quad(const DevParams& dp, const KsArgs& 
     const int lo = max(0, (g0 + j) * alpha - a.base), hi = min(n, (g0 + j + 1) * alpha - a.base);
     const uint32_t* tj = T + ((size_t)(j * ext + t) << dp.log_n);
     const bool own = t >= lo && t < hi;
-    if (a.hoisted) {
+    if (hoisted) {
       // ModUp commutes with the automorphism exactly (centered BConv), so
       // phi(ModUp(a)) is a gather from the ModUp limbs of a. The quads are
       // put in order after the key's loads are under way: in order here, digit
@@ -183,7 +187,7 @@ __device__ __forceinline__ void keymult_quad(const DevParams& dp, const KsArgs& 
     load_vec_stream<4>(e0[j], a.evk + ((size_t)(((g0 + j) * 2 + 0) * ext_top + key_limb) << dp.log_n) + p0);
     load_vec_stream<4>(e1[j], a.evk + ((size_t)(((g0 + j) * 2 + 1) * ext_top + key_limb) << dp.log_n) + p0);
   }
-  if (a.hoisted) {
+  if (hoisted) {
 #pragma unroll
     for (int j = 0; j < D; ++j) src.order(raw[j], x[j]);
   }
@@ -217,7 +221,7 @@ __device__ __forceinline__ void keymult_quad(const DevParams& dp, const KsArgs& 
 template <int D>
 __global__ void k_ks_keymult(DevParams dp, KsArgs a, const uint32_t* T, uint32_t* A, int km_out,
                              uint32_t* km_dst) {
-  keymult_quad<D>(dp, a, T, A, blockIdx.y, stream_pos(), km_out, km_dst, true);
+  keymult_quad<D, true>(dp, a, T, A, blockIdx.y, stream_pos(), km_out, km_dst, true);
 }
 
 static void launch_keymult(int digits, dim3 g, int th, cudaStream_t st, const DevParams& dp, const KsArgs& a,
@@ -885,7 +889,7 @@ __device__ __forceinline__ int load_sys_relaxed(const int* p) {
 template <int D>
 __device__ __forceinline__ void pers_keymult(const DevParams& dp, const PersOp& o, int t) {
   for (uint32_t p0 = 4 * threadIdx.x; p0 < (1u << dp.log_n); p0 += 4 * blockDim.x)
-    keymult_quad<D>(dp, o.ks, o.T, o.A, t, p0, KM_KEYSWITCH, nullptr, false);
+    keymult_quad<D, false>(dp, o.ks, o.T, o.A, t, p0, KM_KEYSWITCH, nullptr, false);
 }
 
 // Element-wise item y = u n + i of HAdd (x + y), PAdd ((x_0 + pt, x_1)) or
