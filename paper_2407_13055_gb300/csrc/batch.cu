@@ -72,10 +72,21 @@ int cuda_fail(ckks_ctx* ctx, cudaError_t e, const char* what) {
   return CKKS_ECUDA;
 }
 
+bool is_key_switch(const ckks_op& o) {
+  return o.op == CKKS_OP_HMULT || o.op == CKKS_OP_HROT || o.op == CKKS_OP_HCONJ;
+}
+
+// Bytes of the limbs that an operation works on: a key switch's inputs and
+// output, ModUp and accumulators (its keys stream past); else inputs and output.
+size_t working_set(const ckks_batch* b, const ckks_op& o, bool key_switch) {
+  const ckks::DevParams& dp = b->ctx->dp;
+  const size_t n = b->ctx->lvl_n(o.a->level), digits = (n + dp.alpha - 1) / dp.alpha;
+  return (6 * n + (key_switch ? (digits + 2) * (n + dp.alpha) : 0)) * 4 << dp.log_n;
+}
+
 // The lane of each operation: in list order, the least loaded of the lanes it
-// may use. An operation may use as many lanes as operations of its level fit
-// in the L2 side by side (the limbs of a key switch: inputs and output, ModUp,
-// accumulators), two at least: above that they push each other's limbs out
+// may use. A key switch may use as many lanes as key switches of its level fit
+// in the L2 side by side, two at least: above that they push each other's limbs out
 // between their kernels, below it more lanes hide more of the launches.
 // 24 operations of one level at N = 2^16, dnum = 3 (us; 1, 2, 4, 6 lanes): level
 // 5 756, 557, 514, 511; level 10 883, 688, 686, 679; level 15 1106, 899, 997,
@@ -83,18 +94,25 @@ int cuda_fail(ckks_ctx* ctx, cudaError_t e, const char* what) {
 // lanes given, lanes in turn -> by this rule: 48 operations of levels 1 .. 39
 // 2866 -> 2602, 33 of levels 10 .. 16 1247 -> 1180, 27 of levels 5 .. 8 660 ->
 // 658 (with 129 MB for the L2 2700, 1194, 662).
+// Other operations beside key switches: by their own limbs where two key switches leave
+// room (12 rescales, 12 HMult at level 10, four lanes: 607 us, as if they were key
+// switches 698), else like key switches (level 20: 1043, 1010). Without a key
+// switch in the batch there is nothing to keep: every lane (24 rescales at
+// level 10, four and eight lanes: 170 and 156 us, on two lanes 239).
 std::vector<int> assign_lanes(const ckks_batch* b) {
-  const ckks::DevParams& dp = b->ctx->dp;
   const size_t nl = b->lanes.size();
+  size_t largest = 0;  // key switch
+  for (const ckks_op& o : b->ops)
+    if (is_key_switch(o)) largest = std::max(largest, working_set(b, o, true));
   std::vector<int> lane(b->ops.size());
   std::vector<size_t> load(nl, 0);  // in 0.6 us at N = 2^16
   for (size_t i = 0; i < b->ops.size(); ++i) {
     const ckks_op& o = b->ops[i];
-    const size_t n = b->ctx->lvl_n(o.a->level), digits = (n + dp.alpha - 1) / dp.alpha;
-    const size_t bytes = (6 * n + (digits + 2) * (n + dp.alpha)) * 4 << dp.log_n;
-    const size_t use = std::min(nl, std::max<size_t>(2, kL2Bytes / bytes));
+    const size_t n = b->ctx->lvl_n(o.a->level);
+    const bool key_switch = is_key_switch(o);
+    const size_t bytes = working_set(b, o, key_switch || 2 * largest > kL2Bytes);
+    const size_t use = largest == 0 ? nl : std::min(nl, std::max<size_t>(2, kL2Bytes / bytes));
     const size_t at = std::min_element(load.begin(), load.begin() + use) - load.begin();
-    const bool key_switch = o.op == CKKS_OP_HMULT || o.op == CKKS_OP_HROT || o.op == CKKS_OP_HCONJ;
     lane[i] = (int)at;
     load[at] += key_switch ? 60 + 4 * n : o.op == CKKS_OP_RESCALE ? 20 + n : 8 + n / 2;
   }
