@@ -27,6 +27,7 @@ struct ckks_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   uint64_t launches_per_run = 0;
+  bool tensor_rescale = true;          // rescalings may take their tensor-core form (see create)
   // persistent form
   bool persistent = false;
   std::vector<int> role;               // per operation: 0 whole on its lane, 1 key switch, 2 element-wise
@@ -46,7 +47,7 @@ namespace {
 
 constexpr size_t kL2Bytes = 100u << 20;  // of 129 MB: the keys stream through the rest
 
-int issue_one(ckks_ctx* lane, const ckks_op& o) {
+int issue_one(const ckks_batch* b, ckks_ctx* lane, const ckks_op& o) {
   switch (o.op) {
     case CKKS_OP_HMULT:
       return ckks_hmult(lane, o.a, o.b, o.evk, o.flags, o.out);
@@ -57,7 +58,7 @@ int issue_one(ckks_ctx* lane, const ckks_op& o) {
     case CKKS_OP_PMULT:
       return ckks_pmult(lane, o.a, o.pt, o.out);
     case CKKS_OP_RESCALE:
-      return ckks_rescale(lane, o.a, o.out);
+      return rescale_op(lane, o.a, o.out, b->tensor_rescale);
     case CKKS_OP_HADD:
       return ckks_hadd(lane, o.a, o.b, o.out);
     case CKKS_OP_PADD:
@@ -131,7 +132,7 @@ int issue_all(ckks_batch* b) {
   const std::vector<int> lane_of = assign_lanes(b);
   for (size_t i = 0; i < b->ops.size(); ++i) {
     ckks_ctx* lane = b->lanes[lane_of[i]];
-    const int rc = issue_one(lane, b->ops[i]);
+    const int rc = issue_one(b, lane, b->ops[i]);
     if (rc != CKKS_OK) {
       if (lane != ctx) ctx->err = lane->err;
       return rc;
@@ -172,7 +173,7 @@ int issue_persistent(ckks_batch* b) {
   for (size_t i = 0; i < b->ops.size() && rc == CKKS_OK; ++i) {
     ckks_ctx* lane = b->lanes[i % nl];
     if (b->role[i] == 0) {
-      rc = issue_one(lane, b->ops[i]);
+      rc = issue_one(b, lane, b->ops[i]);
       if (rc != CKKS_OK && lane != b->ctx) b->ctx->err = lane->err;
     } else if (b->role[i] == 1) {
       ckks::Scratch sc = lane->sc;
@@ -365,6 +366,14 @@ extern "C" int ckks_batch_create(ckks_ctx* ctx, const ckks_op* ops, int count, i
   b->ctx = ctx;
   b->ops.assign(ops, ops + count);
   b->persistent = persistent;
+  // A block of the tensor-core column kernel takes a whole SM, so with four
+  // lanes and nothing larger to run beside, rescalings do better on CUDA cores
+  // (24 of level 30; tensor cores, CUDA cores: two lanes 552, 568 us, four 519,
+  // 470, eight 522, 408; level 20 388, 364; 369, 313; 372, 277; the 25-30
+  // system's level 7 301, 305; 285, 225; 284, 221). Beside key switches,
+  // whose kernels fill the chip, they don't (20 and 4 HRot at level 30 824,
+  // 915).
+  b->tensor_rescale = lanes < 4 || std::any_of(b->ops.begin(), b->ops.end(), is_key_switch);
   // Direct mode: lane 0 is the context itself. Graph mode: every lane is a
   // clone on a private non-blocking stream (stream capture is not possible
   // on the legacy default stream), and the graph is launched into the

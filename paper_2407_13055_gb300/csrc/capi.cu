@@ -1056,25 +1056,28 @@ static double rescale_factor(const ckks_ctx* ctx, int level) {
 }
 
 // Rescale of [2][limbs] at `in` (poly stride sin) from `level` into out.
-static void rescale_into(ckks_ctx* ctx, int level, const uint32_t* in, size_t sin, uint32_t* out, size_t sout) {
-  if (ctx->windowed) launch_rational_rescale(ctx->dp, ctx->sc, ctx->rr[level], in, sin, out, sout, ctx->stream);
-  else launch_rescale(ctx->dp, true, ctx->sc, in, sin, level + 1, out, sout, ctx->stream);
+static void rescale_into(ckks_ctx* ctx, int level, const uint32_t* in, size_t sin, uint32_t* out, size_t sout,
+                         bool tensor = true) {
+  if (ctx->windowed) launch_rational_rescale(ctx->dp, tensor, ctx->sc, ctx->rr[level], in, sin, out, sout, ctx->stream);
+  else launch_rescale(ctx->dp, tensor, ctx->sc, in, sin, level + 1, out, sout, ctx->stream);
 }
 
-int ckks_rescale(ckks_ctx* ctx, const ckks_ct* in, ckks_ct* out) {
+}  // extern "C"
+
+int rescale_op(ckks_ctx* ctx, const ckks_ct* in, ckks_ct* out, bool tensor) {
   if (!ctx || !in || !out) return CKKS_EINVAL;
   if (in->level < 1) return fail(ctx, CKKS_ELEVEL, "rescale at level 0");
   if (out == in || out->d == in->d) return fail(ctx, CKKS_EINVAL, "rescale: output aliases input");
   if (out->cap_level < in->level - 1) return fail(ctx, CKKS_ELEVEL, "rescale: output capacity too small");
   check_ct(ctx, in);
-  rescale_into(ctx, in->level, in->d, in->poly_stride(), out->d, out->poly_stride());
+  rescale_into(ctx, in->level, in->d, in->poly_stride(), out->d, out->poly_stride(), tensor);
   out->level = in->level - 1;
   out->scale = in->scale * rescale_factor(ctx, in->level);
   check_ct(ctx, out);
   return launched(ctx, "rescale");
 }
 
-}  // extern "C"
+extern "C" int ckks_rescale(ckks_ctx* ctx, const ckks_ct* in, ckks_ct* out) { return rescale_op(ctx, in, out, true); }
 
 // Validation and key-switch arguments of HMult (Sec. 2.1: tensor, then
 // relinearization by key switching, then optionally rescaling): fills k,

@@ -653,11 +653,11 @@ __global__ void __launch_bounds__(SL* ColTile<G, TC>::CT) k_rr_cols(DevParams dp
 }
 
 template <class G>
-void launch_rr_cols(const DevParams& dp, const RrArgs& r, const Scratch& sc, cudaStream_t st) {
+void launch_rr_cols(const DevParams& dp, bool tensor, const RrArgs& r, const Scratch& sc, cudaStream_t st) {
   // products per coefficient from which the tensor-core form wins (HMult + rational
   // rescale, levels 1 - 8 of the 25-30 system: 24 products 49.5 against 50.3 us,
   // 30 58.7 / 58.4, 36 65.9 / 65.2, level 8 89.8 / 87.0)
-  if (G::W == 1024 && r.img >= 0 && 2 * r.K * r.n1 >= 30) return launch_rr_tc<G>(dp, r, sc, st);
+  if (tensor && G::W == 1024 && r.img >= 0 && 2 * r.K * r.n1 >= 30) return launch_rr_tc<G>(dp, r, sc, st);
   constexpr int TC = 8, SL = 4;
   const size_t sm = col_smem_bytes<G, TC, SL>(r.K);
   set_col_smem((const void*)k_rr_cols<G, TC, SL>, sm);

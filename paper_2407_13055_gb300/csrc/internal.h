@@ -412,7 +412,7 @@ void launch_hoisted_rotations(const DevParams& dp, const Scratch& sc, const KsAr
                               cudaStream_t st);
 void launch_linear_transform(const DevParams& dp, const Scratch& sc, const KsArgs& a, const LtArgs& lt,
                              cudaStream_t st);
-void launch_rational_rescale(const DevParams& dp, const Scratch& sc, const RrArgs& r, const uint32_t* in,
+void launch_rational_rescale(const DevParams& dp, bool tensor, const Scratch& sc, const RrArgs& r, const uint32_t* in,
                              size_t sin, uint32_t* out, size_t sout, cudaStream_t st);
 // tix: the level whose window is the first n primes, plus one; 0 if no level
 // has that window (then nothing made per level is used).
@@ -420,7 +420,8 @@ void launch_moddown(const DevParams& dp, const Scratch& sc, const uint32_t* acc,
                     cudaStream_t st);
 // Rescale: in [2][n][N] (stride sin) -> out [2][n-1][N] (stride sout).
 // tensor: the column phase may run in its tensor-core form, whose first launch
-// sets a kernel attribute (ckks_rescale_noalloc passes false).
+// sets a kernel attribute (ckks_rescale_noalloc passes false) and whose blocks
+// take whole SMs (some batches pass false).
 void launch_rescale(const DevParams& dp, bool tensor, const Scratch& sc, const uint32_t* in, size_t sin, int n,
                     uint32_t* out, size_t sout, cudaStream_t st);
 
@@ -551,6 +552,8 @@ struct ckks_evk {
   uint32_t galois;
 };
 
+// capi.cu: ckks_rescale; tensor as in launch_rescale.
+int rescale_op(ckks_ctx* ctx, const ckks_ct* in, ckks_ct* out, bool tensor);
 // capi.cu: validation and key-switch arguments of the key-switching
 // operations (out's level and scale are set), shared by the direct calls and
 // the batched forms.

@@ -1175,7 +1175,7 @@ void launch_linear_transform(const DevParams& dp0, const Scratch& sc, const KsAr
 // dropped limb of both polynomials (S = [K][2]), the conversion column
 // kernel (T = [2][n1]), NTT rows with the epilogue. `in` is [2][n0] limbs of
 // the old window (poly stride sin words), `out` [2][n1] of the new one.
-void launch_rational_rescale(const DevParams& dp, const Scratch& sc, const RrArgs& r, const uint32_t* in,
+void launch_rational_rescale(const DevParams& dp, bool tensor, const Scratch& sc, const RrArgs& r, const uint32_t* in,
                              size_t sin, uint32_t* out, size_t sout, cudaStream_t st) {
   CKKS_DISPATCH_LOGN(dp.log_n, {
     prof_mark(sc, st, -1);
@@ -1183,7 +1183,7 @@ void launch_rational_rescale(const DevParams& dp, const Scratch& sc, const RrArg
       // every dropped limb of both polynomials: launch limb y = 2k + u -> S[y]
       launch_rows_inv<G>(dp, SrcDrop{in, sin, r.drop}, sc.S, 2 * r.K, LimbMap{r.rows, 0, 1, 0, 0}, true, st);
       prof_mark(sc, st, P_RS_IN_ROWS);
-      launch_rr_cols<G>(dp, r, sc, st);
+      launch_rr_cols<G>(dp, tensor, r, sc, st);
       prof_mark(sc, st, P_RS_COLS);
     }
     LimbMap m{nullptr, 0, r.n1, r.n1, dp.L};
