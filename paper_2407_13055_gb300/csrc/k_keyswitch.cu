@@ -716,10 +716,12 @@ static int groups_for(int blocks_per_group, int max_groups, int sms) {
 // Streaming grid: four positions per thread. Blocks of 128 threads end and start
 // more evenly than of 256 (HMult + rescale level 39 137.3 -> 136.5 us, the 25-30
 // system's level 6 58.4 -> 57.8, linear transform 329.4 -> 326.4); of 64 they start too
-// slowly (HMult level 20 78.4 -> 83.0).
-static void stream_grid(int log_n, int limbs, dim3& grid, int& threads) {
+// slowly (HMult level 20 78.4 -> 83.0). The transform without a rotated term has
+// little per thread, and there 128 start too slowly (one term at level 39, 256 against
+// 128: 7.5, 11.4 us).
+static void stream_grid(int log_n, int limbs, dim3& grid, int& threads, int most = 128) {
   const int quads = (1 << log_n) / 4;
-  threads = quads < 128 ? quads : 128;
+  threads = quads < most ? quads : most;
   grid = dim3(quads / threads, limbs);
 }
 
@@ -1163,7 +1165,7 @@ void launch_linear_transform(const DevParams& dp0, const Scratch& sc, const KsAr
       prof_mark(sc, st, P_KEYMULT);
       moddown_tail<G>(dp, down, a, sc.A, (size_t)ext * limb, st);
     } else {
-      stream_grid(dp.log_n, 2 * n, g, th);
+      stream_grid(dp.log_n, 2 * n, g, th, 256);
       launch_pdl(dp.pdl, k_lt_plain, g, dim3(th), 0, st, dp, a, lt);
       count_launch(1);
       prof_mark(sc, st, P_KS_EPILOGUE);
