@@ -616,7 +616,7 @@ void launch_cols_tc(const DevParams& dp0, const TcJob& job, int groups, int2 pla
     const TcLayout lay = tc_layout(cap, kr);
     set_col_smem((const void*)k_cols_tc<G, TOP>, lay.total);
     TcPlan pl;
-    std::copy(dp.ks.h_plan + plan.x, dp.ks.h_plan + plan.x + plan.y + 1, pl.at);
+    std::copy(dp.ks.h->plan + plan.x, dp.ks.h->plan + plan.x + plan.y + 1, pl.at);
     launch_pdl(dp.pdl, k_cols_tc<G, TOP>, dim3(plan.y), dim3(kTcThreads), lay.total, st, dp, job, pl, cap, lay);
     count_launch(1);
   }
@@ -639,12 +639,12 @@ static void launch_modup_tc(const DevParams& dp, int n, int base, int tix, int d
     const int g = base / dp.alpha + j;
     const int lo = std::max(0, g * dp.alpha - base), hi = std::min(n, (g + 1) * dp.alpha - base);
     const size_t at = (size_t)tix * dp.dnum + j;
-    job.g[j] = TcGroup{sc.S + ((size_t)lo << dp.log_n), dp.ks.up_cin + dp.ks.h_up_off[at].x,
-                       dp.ks.tc_img + dp.ks.h_up_img[at].x, nullptr, nullptr,
+    job.g[j] = TcGroup{sc.S + ((size_t)lo << dp.log_n), dp.ks.up_cin + dp.ks.h->up_off[at].x,
+                       dp.ks.tc_img + dp.ks.h->up_img[at].x, nullptr, nullptr,
                        sc.T + ((size_t)j * (n + dp.alpha) << dp.log_n), hi - lo, n + dp.alpha - (hi - lo), base + lo, lo,
                        hi - lo};
   }
-  launch_cols_tc<G, false>(dp, job, digits, dp.ks.h_up_plan[tix], s.by_hand, st);
+  launch_cols_tc<G, false>(dp, job, digits, dp.ks.h->up_plan[tix], s.by_hand, st);
 }
 
 // ModDown of both polynomials to the window.
@@ -653,9 +653,9 @@ static void launch_moddown_tc(const DevParams& dp, int n, int base, int tix, con
                               cudaStream_t st) {
   TcJob job{n, base, {}};
   for (int u = 0; u < 2; ++u)
-    job.g[u] = TcGroup{sc.S + ((size_t)u * dp.alpha << dp.log_n), dp.ks.dn_cin, dp.ks.tc_img + dp.ks.h_dn_img[tix].x,
+    job.g[u] = TcGroup{sc.S + ((size_t)u * dp.alpha << dp.log_n), dp.ks.dn_cin, dp.ks.tc_img + dp.ks.h->dn_img[tix].x,
                        nullptr, nullptr, sc.T + ((size_t)u * n << dp.log_n), dp.alpha, n, dp.L, n, 0};
-  launch_cols_tc<G, false>(dp, job, 2, dp.ks.h_dn_plan[tix], s.by_hand, st);
+  launch_cols_tc<G, false>(dp, job, 2, dp.ks.h->dn_plan[tix], s.by_hand, st);
 }
 
 // ModDown fused with rescaling by the top prime.
@@ -664,10 +664,10 @@ static void launch_rs_fused_tc(const DevParams& dp, int n, const Scratch& sc, ui
                                cudaStream_t st) {
   TcJob job{n - 1, 0, {}};
   for (int u = 0; u < 2; ++u)
-    job.g[u] = TcGroup{sc.S + ((size_t)u * dp.alpha << dp.log_n), dp.ks.dn_cin, dp.ks.tc_img + dp.ks.h_rs_img[n].x,
+    job.g[u] = TcGroup{sc.S + ((size_t)u * dp.alpha << dp.log_n), dp.ks.dn_cin, dp.ks.tc_img + dp.ks.h->rs_img[n].x,
                        nullptr, sc.S + ((size_t)(2 * dp.alpha + u) << dp.log_n),
                        T3 + ((size_t)u * (n - 1) << dp.log_n), dp.alpha + 1, n - 1, dp.L, n, 0};
-  launch_cols_tc<G, true>(dp, job, 2, dp.ks.h_rs_plan[n], s.by_hand, st);
+  launch_cols_tc<G, true>(dp, job, 2, dp.ks.h->rs_plan[n], s.by_hand, st);
 }
 
 // ModDown merged into the rescaling (Sec. 6).
@@ -689,7 +689,7 @@ static void launch_rescale_tc(const DevParams& dp, int n, const Scratch& sc, cud
     job.g[u] = TcGroup{sc.S + ((size_t)u << dp.log_n), reinterpret_cast<const uint2*>(&dp.pc[n - 1].ninv),
                        dp.ks.tc_img + dp.ks.one_img, nullptr, nullptr, sc.T + ((size_t)u * (n - 1) << dp.log_n), 1,
                        n - 1, n - 1, n, 0};
-  launch_cols_tc<G, false>(dp, job, 2, dp.ks.h_one_plan[n], false, st);
+  launch_cols_tc<G, false>(dp, job, 2, dp.ks.h->one_plan[n], false, st);
 }
 
 // Rational rescaling: the dropped limbs (S = [K][2]) to the new window.

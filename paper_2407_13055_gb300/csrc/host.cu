@@ -836,24 +836,25 @@ int build_context(ckks_ctx* ctx, const ckks_params* prm) {
   dp.ks.tc_src = reinterpret_cast<const TcSrcRec*>(base + parts[24].off);
   dp.ks.tc_tgt = reinterpret_cast<const TcTgtRec*>(base + parts[25].off);
   ctx->plan = std::move(plan);
-  dp.ks.h_plan = ctx->plan.data();
+  ctx->tc_host.plan = ctx->plan.data();
   ctx->up_plan = std::move(up_plan);
   ctx->dn_plan = std::move(dn_plan);
   ctx->rs_plan = std::move(rs_plan);
-  dp.ks.h_up_plan = ctx->up_plan.data();
-  dp.ks.h_dn_plan = ctx->dn_plan.data();
-  dp.ks.h_rs_plan = ctx->rs_plan.data();
+  ctx->tc_host.up_plan = ctx->up_plan.data();
+  ctx->tc_host.dn_plan = ctx->dn_plan.data();
+  ctx->tc_host.rs_plan = ctx->rs_plan.data();
   ctx->one_plan = std::move(one_plan);
-  dp.ks.h_one_plan = ctx->one_plan.data();
+  ctx->tc_host.one_plan = ctx->one_plan.data();
   dp.ks.one_img = one_img;
   ctx->up_off = std::move(up_off);
   ctx->up_img = std::move(up_img);
   ctx->dn_img = std::move(dn_img);
   ctx->rs_img = std::move(rs_img);
-  dp.ks.h_up_off = ctx->up_off.data();
-  dp.ks.h_up_img = ctx->up_img.data();
-  dp.ks.h_dn_img = ctx->dn_img.data();
-  dp.ks.h_rs_img = ctx->rs_img.data();
+  ctx->tc_host.up_off = ctx->up_off.data();
+  ctx->tc_host.up_img = ctx->up_img.data();
+  ctx->tc_host.dn_img = ctx->dn_img.data();
+  ctx->tc_host.rs_img = ctx->rs_img.data();
+  dp.ks.h = &ctx->tc_host;
   for (int l = 1; l < nlev && ctx->windowed; ++l) {
     RrArgs& r = ctx->rr[l];
     r.drop = reinterpret_cast<const int2*>(base + parts[13].off) + rr_off[l].drop;

@@ -34,6 +34,24 @@ struct TcTgtRec {
 };
 constexpr int kTcMaxBlocks = 192;  // blocks of a tensor-core column kernel (one per SM)
 
+// Host copies (the context's) of the tensor-core form's offsets, for the
+// launchers, behind one pointer: every kernel takes a DevParams by value, and
+// the launch costs time by its size.
+struct TcHost {
+  const int2* up_off;
+  const int2* up_img;
+  const int2* dn_img;
+  const int2* rs_img;
+  // Division of the tensor-core column kernels' work: block boundaries in
+  // plan at (offset, blocks) per conversion (up_plan[tix], dn_plan[tix],
+  // rs_plan[n], one_plan[n], MmArgs::plan, RrArgs::plan).
+  const uint32_t* plan;
+  const int2* up_plan;
+  const int2* dn_plan;
+  const int2* rs_plan;
+  const int2* one_plan;
+};
+
 // Key-switching constants on the device (all built by host.cu).
 struct KsTables {
   // ModUp (Alg. 1 Q_j -> PQ): for the level with n ciphertext limbs and digit
@@ -68,26 +86,14 @@ struct KsTables {
   // conversion matrices in the shared-memory layout of the MMA's B operand,
   // one allocation tc_img; entries (byte offset, bytes) per conversion:
   // up_img[tix * dnum + j] (ModUp digit j), dn_img[tix] (ModDown),
-  // rs_img[n] (fused ModDown + rescale at n limbs), all h_*; MmArgs::img. Null tc_img:
+  // rs_img[n] (fused ModDown + rescale at n limbs), all in TcHost; MmArgs::img. Null tc_img:
   // the tensor-core kernels are not available (more than 16 sources).
   // tc_src, tc_tgt: per prime, its column twiddles and reduction constants.
   const uint8_t* tc_img;
   const TcSrcRec* tc_src;
   const TcTgtRec* tc_tgt;
-  // Host copies (the context's) of the offsets, for the launchers.
-  const int2* h_up_off;
-  const int2* h_up_img;
-  const int2* h_dn_img;
-  const int2* h_rs_img;
   int one_img;  // offset of the one-source image [1]_{q_i}, i < L - 1 (rescaling by one prime)
-  // Division of the tensor-core column kernels' work: block boundaries in
-  // h_plan (host) at (offset, blocks) per conversion (h_up_plan[tix],
-  // h_dn_plan[tix], h_rs_plan[n], h_one_plan[n], MmArgs::plan, RrArgs::plan).
-  const uint32_t* h_plan;
-  const int2* h_up_plan;
-  const int2* h_dn_plan;
-  const int2* h_rs_plan;
-  const int2* h_one_plan;
+  const TcHost* h;  // host
 };
 
 struct DevParams {
@@ -113,6 +119,7 @@ struct DevParams {
   uint32_t* status = nullptr;
   long long wait_limit = 1ll << 32;
 };
+static_assert(sizeof(DevParams) <= 232, "every launch copies it: host-side tables stay behind one pointer");
 
 // Limb -> prime id. Either an explicit device array, or the extended-
 // polynomial rule: limb t (mod per_poly) < n -> q_t, else p_{t - n}.
@@ -209,7 +216,7 @@ struct MmArgs {
   const int32_t* mat;  // [n1][K]: [(P T_drop / s_k) 2^32]_t, centered
   const MmEpi* epi;    // [n1]
   int img;             // byte offset of the matrix's plane image, -1 above 16 sources
-  int2 plan;           // its work division in h_plan
+  int2 plan;           // its work division in TcHost::plan
 };
 
 struct RrArgs {
@@ -496,7 +503,8 @@ struct ckks_ctx {
   std::vector<int> rows_off, rows_cnt;  // per level + 1: ModUp row-table range
   std::vector<ckks::RrArgs> rr;         // per level l >= 1 (windowed): transition l -> l - 1
   std::vector<uint32_t> plan;
-  std::vector<int2> up_off, up_img, dn_img, rs_img, up_plan, dn_plan, rs_plan, one_plan;  // host copies behind dp.ks.h_* (the parent's, for a clone)
+  std::vector<int2> up_off, up_img, dn_img, rs_img, up_plan, dn_plan, rs_plan, one_plan;  // behind tc_host
+  ckks::TcHost tc_host{};  // dp.ks.h (the parent's, for a clone)
   std::vector<ckks::MmArgs> mm;         // per level l >= 1: merged ModDown + rescaling l -> l - 1
   int n_levels() const { return (int)lvl_count.size(); }
   int lvl_n(int level) const { return lvl_count[level]; }
