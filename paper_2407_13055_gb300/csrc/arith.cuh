@@ -79,11 +79,11 @@ __device__ __forceinline__ uint32_t fix_signed(int32_t v, uint32_t q) {
 
 // Harvey-style lazy butterflies with Shoup twiddles (w, wsh).
 // LAZY (q < 2^30): forward inputs/outputs in [0, 4q); inverse in [0, 2q).
-// !LAZY (q < 2^31): forward and inverse values in [0, 2q).
-template <bool LAZY>
+// !LAZY (q < 2^31): forward and inverse values in [0, 2q). ROT: 2q by twice().
+template <bool LAZY, bool ROT = true>
 __device__ __forceinline__ void ct_bfly(uint32_t& x, uint32_t& y, uint32_t w, uint32_t wsh, uint32_t q) {
   if (LAZY) {
-    const uint32_t q2 = twice(q);
+    const uint32_t q2 = ROT ? twice(q) : 2 * q;
     x = csub(x, q2);
     uint32_t t = shoup(y, w, wsh, q);
     y = x - t + q2;

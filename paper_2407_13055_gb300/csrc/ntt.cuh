@@ -30,7 +30,7 @@ struct Log2<1> {
 };
 
 // Forward pass: log2 E Cooley-Tukey stages on E registers.
-template <int E, bool LAZY>
+template <int E, bool LAZY, bool ROT = true>
 __device__ __forceinline__ void ct_pass(uint32_t (&x)[E], const uint2* __restrict__ tw, uint32_t base,
                                         uint32_t q) {
   constexpr int e = Log2<E>::v;
@@ -43,7 +43,7 @@ __device__ __forceinline__ void ct_pass(uint32_t (&x)[E], const uint2* __restric
 #pragma unroll
       for (int r = 0; r < half; ++r) {
         const int i0 = b * 2 * half + r;
-        ct_bfly<LAZY>(x[i0], x[i0 + half], w.x, w.y, q);
+        ct_bfly<LAZY, ROT>(x[i0], x[i0 + half], w.x, w.y, q);
       }
     }
   }
@@ -144,12 +144,12 @@ __device__ __forceinline__ void row_inv(uint32_t (&x)[ER], uint32_t* buf, const 
 }
 
 // Column phase, forward: A layout along h in, B layout out.
-template <int EC, int TC, bool LAZY>
+template <int EC, int TC, bool LAZY, bool ROT = true>
 __device__ __forceinline__ void col_fwd(uint32_t (&x)[EC], uint32_t* buf, const uint2* tw, int jj, int c,
                                         uint32_t q, int bar = 0, int nthr = 0) {
-  ct_pass<EC, LAZY>(x, tw, 1, q);
+  ct_pass<EC, LAZY, ROT>(x, tw, 1, q);
   col_a_to_b<EC, TC>(x, buf, jj, c, bar, nthr);
-  ct_pass<EC, LAZY>(x, tw, EC + jj, q);
+  ct_pass<EC, LAZY, ROT>(x, tw, EC + jj, q);
 }
 
 // Column phase, inverse: B layout in, A layout out.
