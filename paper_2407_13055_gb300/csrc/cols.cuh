@@ -533,13 +533,16 @@ static bool shape_ok(const ColShape& s) {
 // From this many products per coefficient (sources times targets, summed over a
 // launch's conversions) the tensor-core form is the faster one at N = 2^16:
 // below it, a block's start (tensor memory, tables, the first product) costs
-// more than the products it saves. The lines lie where whole operations were
-// equal, levels 0-15, 5 to 15 sources: HRot by the ModUp form at 42 products
-// 39.4 against 40.4 us (CUDA cores first), at 70 43.6 / 43.6, at 112 46.7 /
-// 46.4, at 574 77.7 / 72.8; by the ModDown form at 32 33.5 / 35.8, at 84 40.9 /
-// 40.4, at 196 48.1 / 46.4; HMult + rescale, whose top limb takes a product of
-// its own, at 60 45.5 / 49.6, at 120 51.5 / 52.6, at 210 56.3 / 56.3, at 420
-// 67.3 / 65.1.
+// more than the products it saves. The lines lie where whole operations are
+// about equal (levels 1 to 20, 8 and 14 sources; us, CUDA cores first): HRot by
+// the ModUp form at 40 products 35.4, 35.5, at 42 37.9, 37.1, at 64 38.4, 38.5, at
+// 84 42.3, 40.5, at 196 54.2, 49.0, at 490 73.2, 66.6 (each waited for: at 64
+// 45.3, 48.6, at 84 50.8, 51.3, at 136 55.7, 54.4); by the ModDown form at 56
+// 35.3, 37.1, at 84 38.0, 37.9, at 112 38.7, 38.9, at 140 39.8, 39.4, at 196
+// 43.0, 41.4, at 588 71.9, 66.6; HMult + rescale, whose top limb takes a product
+// of its own, at 60 41.2, 44.4, at 120 44.8, 45.4, at 180 47.6, 48.0, at 210 49.7,
+// 49.0, at 300 54.9, 54.0, at 600 80.4, 75.8; merged with it at 80 41.8, 43.3, at
+// 126 55.6, 55.5, at 182 63.7, 63.0.
 static int tensor_work(ColKernel k) { return k == CK_RS_FUSED ? 200 : 64; }
 
 // The level's tuned shape; else the tensor-core form (N = 2^16, at most 16
@@ -654,10 +657,11 @@ __global__ void __launch_bounds__(SL* ColTile<G, TC>::CT) k_rr_cols(DevParams dp
 
 template <class G>
 void launch_rr_cols(const DevParams& dp, bool tensor, const RrArgs& r, const Scratch& sc, cudaStream_t st) {
-  // products per coefficient from which the tensor-core form wins (HMult + rational
-  // rescale, levels 1 - 8 of the 25-30 system: 24 products 49.5 against 50.3 us,
-  // 30 58.7 / 58.4, 36 65.9 / 65.2, level 8 89.8 / 87.0)
-  if (tensor && G::W == 1024 && r.img >= 0 && 2 * r.K * r.n1 >= 30) return launch_rr_tc<G>(dp, r, sc, st);
+  // products per coefficient from which the tensor-core form wins (levels of the
+  // 25-30 system, us, CUDA cores first; HMult + rational rescale: 24 products 46.1,
+  // 47.4, 28 65.8, 64.5, 30 53.9, 53.8, 36 61.9, 60.6, 52 82.9, 80.3; rescale: 24
+  // 12.1, 14.7, 28 16.6, 15.6, 30 15.4, 15.8, 36 16.3, 15.6, 52 22.0, 19.4)
+  if (tensor && G::W == 1024 && r.img >= 0 && 2 * r.K * r.n1 >= 28) return launch_rr_tc<G>(dp, r, sc, st);
   constexpr int TC = 8, SL = 4;
   const size_t sm = col_smem_bytes<G, TC, SL>(r.K);
   set_col_smem((const void*)k_rr_cols<G, TC, SL>, sm);

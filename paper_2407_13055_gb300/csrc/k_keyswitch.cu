@@ -1221,10 +1221,12 @@ void launch_rescale(const DevParams& dp, bool tensor, const Scratch& sc, const u
     // top limb of both polynomials -> S [2] (compact)
     launch_rows_g<G>(dp, true, in, sc.S, 2, LimbMap{nullptr, top, n, n, dp.L, 1, (int)(sin >> dp.log_n)}, true, st);
     prof_mark(sc, st, P_RS_IN_ROWS);
-    // tensor-core form from 12 targets on (product, sum and rescale at level 13
-    // 31.0 us in either form, 30 53.4 against 60.4, 39 63.7 against 73.8, below
-    // it the start of its blocks shows: level 4 22.7 against 20.6)
-    if (tensor && G::W == 1024 && dp.ks.tc_img && top >= 12) {
+    // tensor-core form from 15 targets on: below, the start of its blocks shows.
+    // CUDA cores, tensor cores (us): rescale at level 12 15.1, 16.0, 14 16.2, 17.9,
+    // 15 18.0, 17.5, 20 20.9, 19.9, 30 29.2, 26.4, 39 36.2, 31.9 (each waited for:
+    // equal at 16 to 22); product, sum and rescale 4 13.6, 15.9, 14 21.6, 22.3, 16
+    // 25.7, 25.5, 20 28.6, 28.3, 30 42.7, 39.6, 39 54.2, 48.9
+    if (tensor && G::W == 1024 && dp.ks.tc_img && top >= 15) {
       launch_rescale_tc<G>(dp, n, sc, st);
     } else {
       const int tiles = G::W / G::TC;
