@@ -137,7 +137,8 @@ int ckks_ctx_clone(ckks_ctx* parent, void* cuda_stream, ckks_ctx** out);
 const char* ckks_last_error(ckks_ctx* ctx);
 int ckks_sync(ckks_ctx* ctx);            /* cudaStreamSynchronize on the context stream */
 void ckks_free(void* handle);            /* any ckks_ct / ckks_pt / ckks_sk / ckks_evk */
-/* Device bytes held by the context's tables and scratch (admission control). */
+/* Device bytes held by the context's tables, scratch and, once it has encoded or
+ * decoded, the workspace that it keeps for that (admission control). */
 size_t ckks_ctx_device_bytes(ckks_ctx* ctx);
 /* Object memory budget (not from the paper: admission control for serving).
  * The device memory of the objects created through a context and its clones

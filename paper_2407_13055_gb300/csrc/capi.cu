@@ -397,7 +397,9 @@ int ckks_sync(ckks_ctx* ctx) {
   return sync_check(ctx, "stream synchronize");
 }
 
-size_t ckks_ctx_device_bytes(ckks_ctx* ctx) { return ctx ? ctx->table_bytes + ctx->scratch_bytes : 0; }
+size_t ckks_ctx_device_bytes(ckks_ctx* ctx) {
+  return ctx ? ctx->table_bytes + ctx->scratch_bytes + ctx->enc_bytes.load() : 0;
+}
 
 }  // extern "C"
 
@@ -862,9 +864,13 @@ int ckks_evk_import(ckks_ctx* ctx, const uint32_t* host, uint32_t galois, ckks_e
 // Workspace of encoding and decoding: N complex values, then N / 2 slots.
 static int enc_workspace(ckks_ctx* ctx) {
   if (ctx->d_enc) return CKKS_OK;
-  const cudaError_t e = cudaMalloc(&ctx->d_enc, (size_t)ctx->N * 3 / 2 * sizeof(double2));
-  if (e != cudaSuccess) ctx->d_enc = nullptr;
-  return e == cudaSuccess ? CKKS_OK : CKKS_ENOMEM;
+  const size_t bytes = (size_t)ctx->N * 3 / 2 * sizeof(double2);
+  if (cudaMalloc(&ctx->d_enc, bytes) != cudaSuccess) {
+    ctx->d_enc = nullptr;
+    return CKKS_ENOMEM;
+  }
+  ctx->enc_bytes += bytes;
+  return CKKS_OK;
 }
 
 // The slots' rounded polynomial modulo the limbs' primes, NTT domain.
@@ -917,12 +923,14 @@ int ckks_decode(ckks_ctx* ctx, const ckks_pt* pt, double* re_im_out) {
   std::lock_guard<std::mutex> lock(ctx->enc_lock);
   if (ctx->dec_limbs < n) {
     if (ctx->d_dec) cudaFree(ctx->d_dec);
+    ctx->enc_bytes -= (size_t)ctx->dec_limbs * limb_words(ctx) * 4;
     ctx->dec_limbs = 0;
     if (cudaMalloc(&ctx->d_dec, bytes) != cudaSuccess) {
       ctx->d_dec = nullptr;
       return fail(ctx, CKKS_ENOMEM, "decode scratch");
     }
     ctx->dec_limbs = n;
+    ctx->enc_bytes += bytes;
   }
   if (enc_workspace(ctx)) return fail(ctx, CKKS_ENOMEM, "decode scratch");
   double2* slots = ctx->d_enc + ctx->N;

@@ -488,6 +488,7 @@ struct ckks_ctx {
   double2* d_enc = nullptr;
   uint32_t* d_dec = nullptr;
   int dec_limbs = 0;
+  std::atomic<size_t> enc_bytes{0};  // of both, read without the lock
   // host-side key-switching constants needed for keygen (gadget P mod prime)
   std::vector<uint2> gadget_p;  // [L + alpha] Shoup pair of [P]_{prime}
   std::string err;
