@@ -134,6 +134,29 @@ def kernel_models(n=L, alpha=ALPHA):
     return out
 
 
+def converted_values(stage, n=L, alpha=ALPHA):
+    """Values per launch that a column stage's BConv makes (targets times N)."""
+    targets = {"modup_cols": sum(n + alpha - a for a in digit_sizes(n, alpha)), "moddown_cols": 2 * n,
+               "rescale_cols": 2 + 2 * (n - 1)}
+    return targets.get(stage, 0) << LOG_N
+
+
+def integer_pipe_work(mdl, converted):
+    """A column stage's model with the BConv on the tensor cores: the integer
+    multiply pipes then do one Shoup product per converted value (its plane
+    sums' residue) in place of the BConv products."""
+    w = dict(mdl, mac=0, shoup=mdl["shoup"] + converted)
+    w["modmul"] = w["shoup"] + w["smr"]
+    return w
+
+
+def lanes_used(lanes, n=L, alpha=ALPHA):
+    """Lanes that a batch's key switches of n limbs share (batch.cu): as many as
+    fit in 100 MiB of the L2 by the limbs they work on, two at least."""
+    limbs = 6 * n + (-(-n // alpha) + 2) * (n + alpha)
+    return min(lanes, max(2, (100 << 20) // (limbs * LIMB_BYTES)))
+
+
 def multiply_costs(rates):
     """SM clocks per modular product of each kind at the measured issue rates
     (instructions per SM per clock of mad.lo, mad.hi, mad.wide)."""
@@ -473,8 +496,8 @@ def run_native(args, rank, world, local_rank):
             K.ckks_hrot(lanes[l], cts[i], 1, gk, outs_r[l])
 
     # the timed step through the batch API: the same 2 x BATCH independent
-    # operations (own outputs), lane l taking HMult and HRot of ciphertexts
-    # i = l mod lanes, issued by the library (direct) or replayed as one CUDA
+    # operations (own outputs), on the lanes that the library gives operations
+    # of this size (lanes_used), issued by it (direct) or replayed as one CUDA
     # graph per step (graph); "python" issues them one call at a time
     batch, outs_b = None, []
     if args.issue != "python":
@@ -596,6 +619,14 @@ def run_native(args, rank, world, local_rank):
         n_ops, ms_op = K.ckks_bench_intop(ctx, op, 4096)
         rates[name] = n_ops / (ms_op * 1e-3) / (sms * clk_hz)
     cost = multiply_costs(rates)
+    # a column stage in its tensor-core form (a tuned shape with 8 or 16 targets
+    # at a time, or the rule's choice at this size) leaves its BConv products to the
+    # tensor cores
+    shape = tuned[LEVEL].get(dom) if tuned else None
+    tensor = converted_values(dom) > 0 and (not shape or shape[0] == 0 or shape[3] >= 8)
+    tensor_products = mdl["mac"] if tensor else 0
+    if tensor:
+        mdl = integer_pipe_work(mdl, converted_values(dom))
     sm_clocks = sum(mdl.get(k, 0) * cost[k] for k in cost)
     alu_peak = mdl["modmul"] / (sm_clocks / (sms * clk_hz)) / 1e12
     alu_ach = mdl["modmul"] / avg_s / 1e12
@@ -604,7 +635,10 @@ def run_native(args, rank, world, local_rank):
            "peak_source": f"derived: {sms} SM x sm_max_mhz / (the kernel's products x SM clocks per product at "
                           "the measured mad.lo / mad.hi / mad.wide issue rates)",
            "int_multiply_per_sm_clk": rates, "algorithmic_modmul_per_launch": mdl["modmul"],
-           "mix": {k: mdl.get(k, 0) for k in ("shoup", "mac", "smr")}, "traffic": ncu_traffic(dom)}
+           "mix": {k: mdl.get(k, 0) for k in ("shoup", "mac", "smr")},
+           "tensor_core_products_per_launch": tensor_products,
+           "note": "products on the integer multiply pipes only; butterfly additions, digits, plane sums and "
+                   "transposes issue beside them", "traffic": ncu_traffic(dom)}
     roof, other = (alu, hbm) if alu["frac"] >= hbm["frac"] else (hbm, alu)
     roof = dict(roof, other={k: other[k] for k in ("bound", "achieved", "peak", "unit", "frac")})
     stage = {k: {"ms_per_launch": (v[0] / v[1] if v[1] else None), "launches": v[1],
@@ -618,8 +652,11 @@ def run_native(args, rank, world, local_rank):
         "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "u32", "data": "synthetic (fresh encryptions of U[-1,1] messages)",
         "config": workload_config({"parallelism": f"replicas{world}",
-                                   "lanes": f"{args.lanes} concurrent CUDA streams (context clones), "
-                                            "independent ciphertexts per lane",
+                                   "lanes": f"{args.lanes} CUDA streams (context clones), independent "
+                                            "ciphertexts; " + (
+                                                f"operations of this size share {lanes_used(args.lanes)} of them "
+                                                "(ckks_batch_create)" if batch is not None
+                                                else "operations on all of them in turn"),
                                    "issue": {"graph": "ckks_batch_run: the step's operations replayed as one "
                                                       "CUDA graph",
                                              "direct": "ckks_batch_run: the library issues the step's "
