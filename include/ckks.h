@@ -191,7 +191,7 @@ int ckks_encode(ckks_ctx* ctx, const double* re_im, int level, double scale, ckk
  * auxiliary primes, stored [level + 1 Q limbs][n_p P limbs]. ckks_pmult and
  * ckks_pt_export use its Q limbs. */
 int ckks_encode_ext(ckks_ctx* ctx, const double* re_im, int level, double scale, ckks_pt** out);
-/* Decode: iNTT on the device, centered CRT lift and FFT on the host; writes
+/* Decode: iNTT, centered CRT lift and FFT (binary64) on the device; writes
  * N/2 interleaved complex slots. Synchronizes. */
 int ckks_decode(ckks_ctx* ctx, const ckks_pt* pt, double* re_im_out);
 /* Eq. 1: (b, a) = (-a s + m + e, a) with a uniform and e Gaussian from the

@@ -60,7 +60,7 @@ constexpr int kTcCap = 56;
 constexpr long long kTcWaitFloor = 1ll << 24;
 constexpr long long kTcDrainLimit = 1ll << 32;
 
-constexpr int kTcWarpgroups = 5, kTcColumns = 16;
+constexpr int kTcColumns = 16;
 constexpr int kTcMaxGroups = 8;  // conversions of a launch (ModUp digits)
 constexpr int kTcMmaWarps = 4;   // one per scheduler
 constexpr int kTcThreads = (kTcWarpgroups * 4 + kTcMmaWarps) * 32;
@@ -627,8 +627,6 @@ extern template void launch_cols_tc<Geo<8, 32>, false>(const DevParams&, const T
 extern template void launch_cols_tc<Geo<8, 32>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
 extern template void launch_cols_tc<Geo<8, 8>, false>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
 extern template void launch_cols_tc<Geo<8, 8>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
-extern template void launch_cols_tc<Geo<4, 4>, false>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
-extern template void launch_cols_tc<Geo<4, 4>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
 
 // ModUp of the level's digits: each to every other prime of the extended basis.
 template <class G>

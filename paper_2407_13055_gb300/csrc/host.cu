@@ -107,7 +107,7 @@ int2 append_planes(std::vector<uint8_t>& img, const int32_t* mat, int ld, int M,
 // boundaries item * 256 + target / 4 appended to plan: (offset, blocks).
 int2 tc_plan(std::vector<uint32_t>& plan, const std::vector<int2>& groups, int tiles, int sms) {
   sms = std::min(sms, kTcMaxBlocks);
-  constexpr int kTcWarpgroups = 5, kStart = 5;
+  constexpr int kStart = 5;
   struct Item {
     int src, quads;
   };

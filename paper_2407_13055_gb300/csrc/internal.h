@@ -33,6 +33,7 @@ struct TcTgtRec {
   uint2 tw[64];
 };
 constexpr int kTcMaxBlocks = 192;  // blocks of a tensor-core column kernel (one per SM)
+constexpr int kTcWarpgroups = 5;   // of a block, which split its sources and targets
 
 // Host copies (the context's) of the tensor-core form's offsets, for the
 // launchers, behind one pointer: every kernel takes a DevParams by value, and

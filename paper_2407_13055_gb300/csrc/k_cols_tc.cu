@@ -7,7 +7,5 @@ template void launch_cols_tc<Geo<8, 32>, false>(const DevParams&, const TcJob&, 
 template void launch_cols_tc<Geo<8, 32>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
 template void launch_cols_tc<Geo<8, 8>, false>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
 template void launch_cols_tc<Geo<8, 8>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
-template void launch_cols_tc<Geo<4, 4>, false>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
-template void launch_cols_tc<Geo<4, 4>, true>(const DevParams&, const TcJob&, int, int2, bool, cudaStream_t);
 
 }  // namespace ckks
