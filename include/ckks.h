@@ -287,8 +287,8 @@ int ckks_linear_transform(ckks_ctx* ctx, const ckks_ct* ct, int count, const int
  * A batch is a list of independent operations (no operation's output may be
  * an input or output of another one in the same batch) issued across `lanes`
  * execution lanes (ckks_ctx_clone) that fork from and join into the context
- * stream; large operations share the first few of them, so that what runs side
- * by side fits in the L2. use_graph is a set of mode flags:
+ * stream; large key switches share the first few of them, so that what runs
+ * side by side fits in the L2. use_graph is a set of mode flags:
  *  CKKS_BATCH_GRAPH: the whole list is captured once into a CUDA graph and
  *    each ckks_batch_run is a single graph launch;
  *  CKKS_BATCH_PERSISTENT: stage-major form with a persistent kernel. Each
